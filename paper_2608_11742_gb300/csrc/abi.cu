@@ -223,7 +223,11 @@ rps_status prepare_row_stats(const rps_logits *logits, const rps_row_list *rows,
     a.warps = grid * (kStatThreads / 32);
     *topk_grid_out = static_cast<int>(std::min<int64_t>((max_rows + kTopkWarps - 1) / kTopkWarps,
                                                          static_cast<int64_t>(dev.sm_count) * 16));
-    a.min_piece = (a.units_per_row + (kMaxPartials - 2) - 1) / (kMaxPartials - 2);
+    // a piece shorter than one ring chunk would cost its record and its ticket
+    // for less than one copy's worth of row
+    a.min_piece = std::max<int64_t>((a.units_per_row + (kMaxPartials - 2) - 1) / (kMaxPartials - 2),
+                                    std::min<int64_t>(a.units_per_row, 32 * kBatch));
+    a.max_ppr = static_cast<int32_t>((a.units_per_row + a.min_piece - 1) / a.min_piece);
     a.err = dev.err;
     *grid_out = grid;
     return RPS_OK;

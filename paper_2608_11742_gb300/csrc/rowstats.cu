@@ -6,10 +6,11 @@
 //
 // Work split. One block of kStatThreads per SM; each warp streams one piece. With
 // at least as many warps as rows, each row is cut into equal pieces, so that no
-// piece crosses a row boundary; otherwise the rows' 16-byte units are laid end
-// to end and cut into equal contiguous pieces (a piece covers the tail of one
-// row, whole rows and the head of another). Either way every warp streams about
-// the same number of bytes. Each (warp, row) pair leaves a partial record in the
+// piece crosses a row boundary (spread over the blocks when the rows are few);
+// otherwise the rows' 16-byte units are laid end to end and cut into equal
+// contiguous pieces (a piece covers the tail of one row, whole rows and the head
+// of another). Either way every warp streams about the same number of bytes.
+// Each (warp, row) pair leaves a partial record in the
 // workspace and the last warp to finish a row (atomic ticket, no waiting) merges
 // the at most kMaxPartials records and writes the row.
 //
@@ -715,22 +716,39 @@ __device__ __forceinline__ void locate(const RowStatsArgs &a, const int32_t *seg
     describe<DT>(a, seg, s);
 }
 
+// a / b for 0 < b and a below 2^22, exact: the approximate quotient is off by at
+// most one, and the remainder says which way. A fifth of the instructions of an
+// integer division; the 32 warps of a block all compute the cut, in the same
+// issue slots, before the first copy can start.
+__device__ __forceinline__ int div_small(int a, int b) {
+    int q = __float2int_rz(__fdividef(static_cast<float>(a), static_cast<float>(b)));
+    const int r = a - q * b;
+    q += r >= b;
+    q -= r < 0;
+    return q;
+}
+
 // The cut of the rows' units into pieces, one per warp. Aligned: each row is
-// cut into equal pieces (at most ceil(nv / min_piece) per row), so that no
-// piece crosses a row boundary, where a warp's stream stops for the row's
-// record; taken when it leaves at most an eighth of the warps idle. Otherwise
-// all units are cut evenly (pieces of at least min_piece units). Returns the
-// units per piece.
-__device__ __forceinline__ int64_t piece_units(const RowStatsArgs &a, int64_t total_rows, int64_t nv,
-                                               bool &aligned) {
-    aligned = false;
-    if (total_rows <= a.warps) {  // 32-bit arithmetic: rows, warps and units of a row fit
-        const int rows = static_cast<int>(total_rows), n = static_cast<int>(nv), mp = static_cast<int>(a.min_piece);
-        const int ppr = min(a.warps / rows, (n + mp - 1) / mp);
-        const int piece = (n + ppr - 1) / ppr;
-        const int cpr = (n + piece - 1) / piece;
-        if (8 * static_cast<int64_t>(rows) * cpr >= 7 * static_cast<int64_t>(a.warps)) {
-            aligned = true;
+// cut into `cpr` equal pieces (at most a.max_ppr), so that no piece crosses a
+// row boundary, where a warp's stream stops for the row's record. Taken when it
+// leaves at most an eighth of the warps idle, or when the rows are so few that
+// each is cut into max_ppr pieces (the even cut would then have pieces of the
+// same length, and as many idle warps). Otherwise all units are cut evenly, in
+// pieces of at least min_piece units, and cpr is 0. few: each row is in max_ppr
+// pieces, and warps may be left over. Returns the units per piece.
+__device__ __forceinline__ int64_t piece_units(const RowStatsArgs &a, int64_t total_rows, int64_t nv, int &cpr,
+                                               bool &few) {
+    cpr = 0;
+    few = false;
+    if (total_rows <= a.warps && nv < (1 << 21) && a.warps < (1 << 21)) {
+        const int rows = static_cast<int>(total_rows), n = static_cast<int>(nv);
+        const int per = div_small(a.warps, rows);
+        const int ppr = min(per, a.max_ppr);
+        const int piece = div_small(n + ppr - 1, ppr);
+        const int c = div_small(n + piece - 1, piece);
+        if (ppr == a.max_ppr || 8 * rows * c >= 7 * a.warps) {
+            cpr = c;
+            few = ppr == a.max_ppr;
             return piece;
         }
     }
@@ -862,7 +880,6 @@ __global__ void __launch_bounds__(kStatThreads, kStatBlocksPerSm) row_stats_kern
     pdl_launch_next();
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
-    const int warp = blockIdx.x * kWarps + wib;
     uint4 *ring = dyn + wib * (kRing * kChunkUnits);
     uint64_t *bar = bars[wib];
 
@@ -879,23 +896,28 @@ __global__ void __launch_bounds__(kStatThreads, kStatBlocksPerSm) row_stats_kern
     const int64_t nv = a.units_per_row;
     const int64_t total = total_rows * nv;
     if (total == 0) return;
-    // With at least as many warps as rows, each row is cut into equal pieces
-    // (aligned: no piece crosses a row boundary, where a warp's stream would
-    // stop for the row's record); otherwise the units are cut evenly.
-    __shared__ int64_t cut_cpr[kWarps];  // pieces per row of an aligned cut, 0 for the even cut
-    if (lane == 0) cut_cpr[wib] = 0;
-    bool aligned = false;
-    const int64_t piece = piece_units(a, total_rows, nv, aligned);
+    __shared__ int cut_cpr[kWarps];  // pieces per row of an aligned cut, 0 for the even cut
+    int cpr0;
+    bool few;
+    const int64_t piece = piece_units(a, total_rows, nv, cpr0, few);
+    const bool aligned = cpr0 > 0;
+    // With few rows the piece numbers go round the blocks, so that the pieces
+    // spread over every SM instead of filling the first blocks: 32 rows of
+    // 126,464 bf16 logits (960 pieces) held 30 of 152 SMs, which were bound by
+    // their issue slots, and the step of one such block took 56.2 us against
+    // 45.0 spread. With (nearly) all warps in use neighbouring pieces stay in
+    // one block: spread, the 256-position step was 1.2 % slower.
+    const int warp = few ? wib * static_cast<int>(gridDim.x) + static_cast<int>(blockIdx.x)
+                         : static_cast<int>(blockIdx.x) * kWarps + wib;
+    if (lane == 0) cut_cpr[wib] = cpr0;
     if (SKETCH && blockIdx.x == 0 && threadIdx.x == 0) *a.sketch_piece = static_cast<int>(min(piece, nv));
     Walk w0;
     if (aligned) {  // (32-bit: piece and the pieces per row are below the row length)
-        const int cpr = (static_cast<int>(nv) + static_cast<int>(piece) - 1) / static_cast<int>(piece);
-        const int row0 = warp / cpr, part = warp - row0 * cpr;
+        const int row0 = div_small(warp, cpr0), part = warp - row0 * cpr0;
         if (row0 >= total_rows) return;
         w0.r = row0;
         w0.u = part * static_cast<int>(piece);
         w0.left = min(piece, nv - w0.u);
-        if (lane == 0) cut_cpr[wib] = cpr;
     } else {
         const int64_t g_begin = static_cast<int64_t>(warp) * piece;
         if (g_begin >= total) return;
@@ -1015,10 +1037,10 @@ __global__ void __launch_bounds__(kStatThreads, kStatBlocksPerSm) row_stats_kern
         int64_t w_first;
         int count;
         // (read back from shared memory so that it is not kept live through the stream)
-        const int64_t cpr = *reinterpret_cast<volatile int64_t *>(&cut_cpr[wib]);
+        const int cpr = *reinterpret_cast<volatile int *>(&cut_cpr[wib]);
         if (cpr > 0) {
             w_first = r * cpr;
-            count = static_cast<int>(cpr);
+            count = cpr;
         } else {
             w_first = (r * nv) / piece;
             count = static_cast<int>(((r + 1) * nv - 1) / piece - w_first + 1);

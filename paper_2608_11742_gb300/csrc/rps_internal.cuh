@@ -83,6 +83,7 @@ struct RowStatsArgs {
     int64_t units_per_row;
     int32_t warps;
     int64_t min_piece;    // at least ceil(units_per_row / (kMaxPartials - 1))
+    int32_t max_ppr;      // ceil(units_per_row / min_piece): pieces a row is cut into at most
     uint32_t *err;
 };
 
