@@ -26,7 +26,7 @@ LIBS = {
     "librps.so": ["abi.cu", "rowstats.cu", "decide.cu", "decode.cu", "gather.cu", "static_scratch.cu", "lmhead.cu", "attention.cu"],
     "librps_synth.so": ["synth.cu"],
 }
-HEADERS = [INCLUDE / "rps.h", INCLUDE / "rps_synth.h", CSRC / "rps_internal.cuh", CSRC / "umma_desc.h"]
+HEADERS = sorted([*INCLUDE.glob("*.h"), *CSRC.glob("*.h"), *CSRC.glob("*.cuh")])
 
 
 def _stale(target: Path, sources) -> bool:

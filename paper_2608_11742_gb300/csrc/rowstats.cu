@@ -50,6 +50,7 @@
 #include <climits>
 
 #include "rps_internal.cuh"
+#include "topk_device.cuh"
 
 namespace rps {
 namespace {
@@ -58,7 +59,6 @@ constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 constexpr float kSlack = 8.0f;          // nats the reference may trail the maximum
 constexpr int kChunkUnits = 32 * kBatch;  // 16-byte units per ring buffer (2 KB)
-constexpr int kCandBatch = 32;  // top-k candidates merged at a time
 constexpr uint64_t kWaitLimitNs = 200ull * 1000 * 1000;  // a bulk copy normally lands within microseconds
 constexpr uint32_t kUnhealthy = 1u;  // health word of a workspace a launch gave up on
 
@@ -397,11 +397,6 @@ __device__ void rescan_safe(LaneState &L, const char *row, int V, int u0, int u1
 }
 
 // ---------------------------------------------------------------- top-k
-// True when (av, ai) ranks before (bv, bi): larger logit, then lower token id.
-__device__ __forceinline__ bool ranks_before(float av, int ai, float bv, int bi) {
-    return av > bv || (av == bv && ai < bi);
-}
-
 // Insert a warp-uniform candidate into the warp's sorted list (lane j = rank j).
 __device__ __forceinline__ void topk_insert(float &tv, int &ti, float cv, int ci, int k, int lane) {
     const unsigned keep = (k >= 32) ? kFull : ((1u << k) - 1u);
@@ -415,79 +410,6 @@ __device__ __forceinline__ void topk_insert(float &tv, int &ti, float cv, int ci
     } else if (lane > pos) {
         tv = uv;
         ti = ui;
-    }
-}
-
-// k-th largest of the 32 lane values (bitonic sort, descending), 1 <= k <= 32.
-__device__ __forceinline__ float warp_kth_largest(float x, int k, int lane) {
-#pragma unroll
-    for (int size = 2; size <= 32; size <<= 1) {
-#pragma unroll
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            const float o = __shfl_xor_sync(kFull, x, stride);
-            const bool keep_max = ((lane & size) == 0) == ((lane & stride) == 0);
-            x = keep_max ? fmaxf(x, o) : fminf(x, o);
-        }
-    }
-    return __shfl_sync(kFull, x, k - 1);
-}
-
-// Merges one candidate per lane (sentinel -inf / INT_MAX for none) into the
-// warp-distributed sorted list: bitonic sort of the 32 candidates in rank order,
-// then the element-wise better of the list and the reversed candidates (the 32
-// best of both, as a bitonic sequence), then a bitonic merge. Fixed cost,
-// independent of how many candidates are real.
-__device__ __forceinline__ void pair_step(float &v, int &i, int stride, bool keep_better) {
-    const float ov = __shfl_xor_sync(kFull, v, stride);
-    const int oi = __shfl_xor_sync(kFull, i, stride);
-    if (keep_better == ranks_before(ov, oi, v, i)) {
-        v = ov;
-        i = oi;
-    }
-}
-
-// The list holds nothing yet: each real candidate's rank among the 32 is the
-// count of candidates before it (candidates are distinct, so ranks are); ranks
-// below k go to buf[rank] (kCandBatch entries), then lane j takes rank j.
-// Independent shuffles instead of a sorting network's dependent stages.
-__device__ __forceinline__ void warp_rank_into_list(float &tv, int &ti, float cv, int ci, int k, int lane,
-                                                    float2 *buf) {
-    const bool real = ci != INT_MAX;
-    int rank = 0;
-#pragma unroll
-    for (int j = 0; j < 32; ++j) {
-        const float ov = __shfl_sync(kFull, cv, j);
-        const int oi = __shfl_sync(kFull, ci, j);
-        rank += ranks_before(ov, oi, cv, ci);
-    }
-    const int n = __popc(__ballot_sync(kFull, real));
-    __syncwarp();
-    if (real && rank < k) buf[rank] = make_float2(cv, __int_as_float(ci));
-    __syncwarp();
-    const float2 e = lane < k && lane < n ? buf[lane] : make_float2(-INFINITY, __int_as_float(INT_MAX));
-    tv = e.x;
-    ti = __float_as_int(e.y);
-    __syncwarp();
-}
-
-__device__ __forceinline__ void warp_merge_batch(float &tv, int &ti, float cv, int ci, int k, int lane) {
-#pragma unroll
-    for (int size = 2; size <= 32; size <<= 1) {
-#pragma unroll
-        for (int stride = size >> 1; stride > 0; stride >>= 1)
-            pair_step(cv, ci, stride, ((lane & size) == 0) == ((lane & stride) == 0));
-    }
-    const float rv = __shfl_sync(kFull, cv, 31 - lane);
-    const int ri = __shfl_sync(kFull, ci, 31 - lane);
-    if (ranks_before(rv, ri, tv, ti)) {
-        tv = rv;
-        ti = ri;
-    }
-#pragma unroll
-    for (int stride = 16; stride > 0; stride >>= 1) pair_step(tv, ti, stride, (lane & stride) == 0);
-    if (lane >= k) {
-        tv = -INFINITY;
-        ti = INT_MAX;
     }
 }
 
@@ -1106,6 +1028,13 @@ __global__ void __launch_bounds__(kStatThreads, kStatBlocksPerSm) row_stats_kern
 // read again, and their elements at or above it enter the warp-distributed
 // sorted list (lane j = rank j, logit desc then token asc).
 constexpr int kCellCap = 256;  // candidate cells a warp buffers before reloading them
+// Up to this k the bound is taken over one maximum per lane. The vectors that
+// reach it number about 32 ln(32 / (32 - k)): 22 at k = 16, but 44 at k = 24 and
+// over 130 at k = 32, each batch of 32 cells being one reload and one merge of
+// the chain. With two maxima per lane, 288 rows of 32,003 fp32 logits at k = 32:
+// the step 95.5 -> 74.2 us (this launch about 36 -> 15); k <= 16 keeps the
+// shorter chain (one sort).
+constexpr int kOneMaxK = 16;
 constexpr int kSketchVecs = 24;  // 16-byte sketch loads a lane keeps in flight (up to 768 vectors a slot in one round)
 static_assert(kSketchVecs <= 32, "one hit bit per vector");
 
@@ -1285,15 +1214,20 @@ __global__ void __launch_bounds__(kTopkWarps * 32, kTopkMinBlocks) topk_rows_ker
         const SketchRow cut = sketch_row(min(max(__float_as_int(nrm.w), 1), n_units), min(max(piece, 1), n_units),
                                          full_units);
         // the k-th largest of the lanes' largest entries
-        float lane_max = -INFINITY;
+        // (for long lists, of each lane's two largest vectors' maxima)
+        float lane_max = -INFINITY, lane_2nd = -INFINITY;
         for (int v0 = 0;;) {
 #pragma unroll
-            for (int q = 0; q < kSketchVecs; ++q) lane_max = fmaxf(lane_max, vm[q]);
+            for (int q = 0; q < kSketchVecs; ++q) {
+                lane_2nd = fmaxf(lane_2nd, fminf(lane_max, vm[q]));
+                lane_max = fmaxf(lane_max, vm[q]);
+            }
             v0 += 32 * kSketchVecs;
             if (v0 >= n_vec) break;
             vector_maxima<DT>(vm, sk, v0, n_vec, lane);
         }
-        const float theta = warp_kth_largest(lane_max, k, lane);
+        const float theta = k > kOneMaxK ? warp_kth_largest2(lane_max, lane_2nd, k, lane)
+                                         : warp_kth_largest(lane_max, k, lane);
 
         // Pass 2: the cells that reach it, buffered and reloaded kCellCap at a
         // time. Few vectors hold one; only those are read again (from L1).

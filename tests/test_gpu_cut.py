@@ -40,3 +40,25 @@ def test_cut(n, V, bf16, k):
         rps.rps_score_step(t, None, None, 1, n, prm, out, ws, mask_pos=pos)
     assert rps.rps_poll_device_status() == (rps.RPS_OK, 0)
     compare_stats(stats_np(out), oracle_default().row_stats(host[0, 0], k), np.arange(n), k, f"{n} x {V}")
+
+
+@pytest.mark.parametrize("k", [16, 17, 31, 32])
+@pytest.mark.parametrize("kind", ["spread", "equal", "few"])
+def test_long_lists(kind, k):
+    """The bound of long lists (two maxima per lane): spread rows, rows of equal
+    logits, and rows of fewer finite logits than k."""
+    rng = np.random.default_rng(k)
+    n, V = 9, 32003
+    z = np.zeros((1, 1, n, V), np.float32)
+    if kind == "spread":
+        z[:] = rng.standard_normal(z.shape)
+    elif kind == "few":
+        z[:] = -np.inf
+        z[0, 0, :, rng.choice(V, k - 3, replace=False)] = rng.standard_normal((k - 3, n)).astype(np.float32)
+    t = padded_tensor(z)
+    out = rps.RowStatsBuf.alloc(n, k, "cuda")
+    ws = torch.zeros(rps.rps_workspace_bytes(n, V, k, t.dtype), dtype=torch.uint8, device="cuda")
+    rps.rps_score_step(t, None, None, 1, n, configs.Params(k_max=k), out, ws,
+                       mask_pos=torch.arange(n, dtype=torch.int32, device="cuda"))
+    assert rps.rps_poll_device_status() == (rps.RPS_OK, 0)
+    compare_stats(stats_np(out), oracle_default().row_stats(z[0, 0], k), np.arange(n), k, f"{kind} k={k}")
