@@ -44,6 +44,7 @@
 #include <mutex>
 
 #include "rps_internal.cuh"
+#include "topk_device.cuh"
 #include "umma_desc.h"
 
 namespace rps {
@@ -62,7 +63,7 @@ constexpr int kEpiWarps = 4;
 constexpr uint32_t kTmemCols = 2 * kTileN;  // two accumulators
 constexpr int kMaxSplits = 256;
 constexpr int kSmemBytes = kStages * kStageBytes + 1024;  // + slack to align the ring to 1024 bytes
-constexpr int kMergeThreads = 256;
+constexpr int kMergeThreads = 128;
 constexpr uint64_t kDrainNs = 200ull * 1000 * 1000;
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
@@ -492,15 +493,41 @@ __global__ void __launch_bounds__(kThreads, 1)
 }
 
 // ---------------------------------------------------------------- merge
-__device__ __forceinline__ bool better(float v, int i, float w, int j) { return v > w || (v == w && i < j); }
+// One warp per row: the splits' records give zmax, lse, H, P^max and argmax; in
+// top-k mode the splits' sorted lists give T_i, mu and the truncated entropy
+// (Eq. 3). Lane l owns splits l, l + 32, ...
+//
+// Latency bound: a few hundred bytes to 20 KB per row, one chain of dependent
+// round trips, so the chain is kept to two. The records come in one round, and
+// bound the row's k-th logit from below: of the splits' (t + 1)-th logits,
+// t = (k - 1) / splits, the m-th largest with m (t + 1) >= k is reached by m
+// lists of t + 1 logits each. Only lists whose largest logit reaches the bound
+// (about k of them) are read, all their entries at once, and the entries that
+// reach it are ranked by shuffles. V 126,464, k = 10, LM head and merge: 32 rows
+// (152 splits) 213.6 -> 184.6 us, 256 rows (76 splits) 258.4 -> 244.8, against a
+// merge that took one round of loads and shuffles per rank (19 and 13 us alone).
+constexpr int kMergeCand = 256;   // candidates buffered per row before they are ranked
+constexpr int kMergeLoads = 4;    // list loads a lane keeps in flight
 
-// One warp per row: the splits' records give zmax, lse, H, P^max and argmax;
-// in top-k mode a k-way merge of the splits' sorted lists gives T_i, mu and
-// the truncated entropy (Eq. 3). Lane l owns splits l, l + 32, ...
+// Ranks the n buffered candidates into the warp's list, 32 at a time.
+__device__ __forceinline__ void rank_candidates(float &tv, int &ti, const float2 *buf, int n, int k, int lane,
+                                                float2 *scratch, bool &empty) {
+    for (int b = 0; b < n; b += kCandBatch) {
+        const float2 e = b + lane < n ? buf[b + lane] : make_float2(-INFINITY, __int_as_float(INT_MAX));
+        if (empty) warp_rank_into_list(tv, ti, e.x, __float_as_int(e.y), k, lane, scratch);
+        else warp_merge_batch(tv, ti, e.x, __float_as_int(e.y), k, lane);
+        empty = false;
+    }
+    __syncwarp();
+}
+
 template <int KMAX>
 __global__ void __launch_bounds__(kMergeThreads) lmhead_merge_kernel(const LmArgs a) {
     constexpr int kPerLane = kMaxSplits / 32;
-    __shared__ int head_all[kMergeThreads / 32][kMaxSplits];
+    constexpr int kWarps = kMergeThreads / 32;
+    __shared__ int16_t hit_all[KMAX > 0 ? kWarps : 1][kMaxSplits];
+    __shared__ float2 cand_all[KMAX > 0 ? kWarps : 1][kMergeCand + 64];
+    __shared__ float2 scratch_all[KMAX > 0 ? kWarps : 1][kCandBatch];
     pdl_wait();
     pdl_launch_next();
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -508,32 +535,48 @@ __global__ void __launch_bounds__(kMergeThreads) lmhead_merge_kernel(const LmArg
         if (blockIdx.x == 0 && threadIdx.x == 0) flag_error(a.err, RPS_DEVERR_WORKSPACE);
         return;
     }
-    int *head = head_all[wib];
-    const int warps = gridDim.x * (kMergeThreads / 32);
-    for (int row = blockIdx.x * (kMergeThreads / 32) + wib; row < a.n_rows; row += warps) {
+    const int warps = gridDim.x * kWarps;
+    for (int row = blockIdx.x * kWarps + wib; row < a.n_rows; row += warps) {
         const LmPartial *pr = a.part + static_cast<int64_t>(row) * a.splits;
+        const float2 *ls = a.lists + static_cast<int64_t>(row) * a.splits * KMAX;
+        const int t = KMAX > 0 && a.k > 0 ? (a.k - 1) / a.splits : 0;  // depth of the bound (below KMAX: k <= KMAX)
+        float4 p[kPerLane];   // B, s, t, largest logit
+        int pam[kPerLane];
+        float deep[kPerLane]; // the (t + 1)-th logit
+#pragma unroll
+        for (int m = 0; m < kPerLane; ++m) {
+            const int j = lane + 32 * m;
+            p[m] = make_float4(-INFINITY, 0.f, 0.f, -INFINITY);
+            pam[m] = INT_MAX;
+            deep[m] = -INFINITY;
+            if (j < a.splits) {
+                p[m] = *reinterpret_cast<const float4 *>(pr + j);
+                pam[m] = pr[j].amax;
+                if (KMAX > 0 && t > 0) deep[m] = ls[j * KMAX + t].x;
+            }
+        }
         // the largest reference of the row's live records
         float M = -INFINITY, mx = -INFINITY;
         int am = INT_MAX;
         bool nan = false;
-        for (int j = lane; j < a.splits; j += 32) {
-            const LmPartial p = pr[j];
-            if (p.s > 0.f) M = fmaxf(M, p.B);
-            if (p.s != p.s) nan = true;
-            if (p.mx > mx || (p.mx == mx && p.amax < am)) {
-                mx = p.mx;
-                am = p.amax;
+#pragma unroll
+        for (int m = 0; m < kPerLane; ++m) {
+            if (p[m].y > 0.f) M = fmaxf(M, p[m].x);
+            if (p[m].y != p[m].y) nan = true;
+            if (p[m].w > mx || (p[m].w == mx && pam[m] < am)) {
+                mx = p[m].w;
+                am = pam[m];
             }
         }
         M = warp_max(M);
         float S = 0.f, T = 0.f;
-        for (int j = lane; j < a.splits; j += 32) {
-            const LmPartial p = pr[j];
-            if (p.s > 0.f) {
-                const float dl = p.B - M;
+#pragma unroll
+        for (int m = 0; m < kPerLane; ++m) {
+            if (p[m].y > 0.f) {
+                const float dl = p[m].x - M;
                 const float f = ex2(dl);
-                S = fmaf(f, p.s, S);
-                T = fmaf(f, fmaf(dl, p.s, p.t), T);
+                S = fmaf(f, p[m].y, S);
+                T = fmaf(f, fmaf(dl, p[m].y, p[m].z), T);
             }
         }
         S = warp_sum(S);
@@ -560,57 +603,64 @@ __global__ void __launch_bounds__(kMergeThreads) lmhead_merge_kernel(const LmArg
         }
         if constexpr (KMAX > 0) {  // (the statistics-only form has no lists)
             if (a.k == 0) continue;
-            // k-way merge: rank r goes to lane r
-            for (int j = lane; j < a.splits; j += 32) head[j] = 0;
+            int16_t *hit = hit_all[wib];
+            float2 *cand = cand_all[wib];
+            float2 *scratch = scratch_all[wib];
+            // the bound: the m-th largest of the lanes' largest (t + 1)-th logits
+            float dmax = -INFINITY;
+#pragma unroll
+            for (int m = 0; m < kPerLane; ++m) dmax = fmaxf(dmax, t > 0 ? deep[m] : p[m].w);
+            const float theta = warp_kth_largest(dmax, (a.k + t) / (t + 1), lane);
+            int n_hit = 0;
+#pragma unroll
+            for (int m = 0; m < kPerLane; ++m) {
+                const bool h = lane + 32 * m < a.splits && p[m].w >= theta;
+                const unsigned hm = __ballot_sync(kFull, h);
+                if (h) hit[n_hit + __popc(hm & ((1u << lane) - 1u))] = static_cast<int16_t>(lane + 32 * m);
+                n_hit += __popc(hm);
+            }
             __syncwarp();
-            const float2 *ls = a.lists + static_cast<int64_t>(row) * a.splits * KMAX;
             float tv = -INFINITY;
             int ti = INT_MAX;
-            for (int r = 0; r < a.k; ++r) {
-                float bv = -INFINITY;
-                int bi = INT_MAX, bj = -1;
-    #pragma unroll
-                for (int m = 0; m < kPerLane; ++m) {
-                    const int j = lane + 32 * m;
-                    if (j < a.splits && head[j] < KMAX) {
-                        const float2 e = ls[j * KMAX + head[j]];
-                        const int id = __float_as_int(e.y);
-                        if (bj < 0 || better(e.x, id, bv, bi)) {
-                            bv = e.x;
-                            bi = id;
-                            bj = j;
-                        }
+            bool empty = true;
+            int pending = 0;
+            const int items = n_hit * (KMAX / 2);  // two entries each
+            for (int i0 = 0; i0 < items; i0 += 32 * kMergeLoads) {
+                float4 e[kMergeLoads];
+#pragma unroll
+                for (int u = 0; u < kMergeLoads; ++u) {
+                    const int i = i0 + u * 32 + lane;
+                    e[u] = make_float4(-INFINITY, __int_as_float(INT_MAX), -INFINITY, __int_as_float(INT_MAX));
+                    if (i < items)
+                        e[u] = reinterpret_cast<const float4 *>(ls + hit[i / (KMAX / 2)] * KMAX)[i % (KMAX / 2)];
+                }
+#pragma unroll
+                for (int u = 0; u < kMergeLoads; ++u) {
+#pragma unroll
+                    for (int half = 0; half < 2; ++half) {
+                        const float v = half ? e[u].z : e[u].x;
+                        const float id = half ? e[u].w : e[u].y;
+                        const bool in = v >= theta && __float_as_int(id) != INT_MAX;
+                        const unsigned im = __ballot_sync(kFull, in);
+                        if (in) cand[pending + __popc(im & ((1u << lane) - 1u))] = make_float2(v, id);
+                        pending += __popc(im);
+                    }
+                    __syncwarp();
+                    if (pending >= kMergeCand) {
+                        rank_candidates(tv, ti, cand, pending, a.k, lane, scratch, empty);
+                        pending = 0;
                     }
                 }
-                // warp-wide best (logit desc, token asc)
-                float wv = bv;
-                int wi = bi, wl = bj < 0 ? INT_MAX : lane;
-    #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    const float ov = __shfl_xor_sync(kFull, wv, o);
-                    const int oi = __shfl_xor_sync(kFull, wi, o);
-                    const int ol = __shfl_xor_sync(kFull, wl, o);
-                    if (ol != INT_MAX && (wl == INT_MAX || better(ov, oi, wv, wi))) {
-                        wv = ov;
-                        wi = oi;
-                        wl = ol;
-                    }
-                }
-                if (lane == wl) ++head[bj];
-                if (lane == r) {
-                    tv = wl == INT_MAX ? -INFINITY : wv;
-                    ti = wl == INT_MAX ? INT_MAX : wi;
-                }
-                __syncwarp();
             }
+            rank_candidates(tv, ti, cand, pending, a.k, lane, scratch, empty);
             // mu and the truncated entropy against the row's reference, as the streaming kernel forms them
-            float p = 0.f, h = 0.f;
+            float pr_v = 0.f, h = 0.f;
             if (ok && lane < a.k && ti != INT_MAX) {
                 const float u = fmaf(tv, kLog2e, -M);
-                p = ex2(u) * invS;
-                if (p > 0.f) h = -p * (u * kLn2 - lnS);
+                pr_v = ex2(u) * invS;
+                if (pr_v > 0.f) h = -pr_v * (u * kLn2 - lnS);
             }
-            const float mu = warp_sum(p), ht = warp_sum(h);
+            const float mu = warp_sum(pr_v), ht = warp_sum(h);
             if (lane == 0) {
                 a.mu[row] = ok ? mu : NAN;
                 a.htrunc[row] = ok ? ht : NAN;

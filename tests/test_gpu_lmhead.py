@@ -78,6 +78,18 @@ def check(h_bits, w_bits, k, rows=None):
     return err.max()
 
 
+@pytest.mark.parametrize("n,V,k,zero", [
+    (1300, 9000, 20, 0),   # 13 splits for 20 ranks: the bound is taken two entries deep
+    (5, 300, 32, 0),       # two splits: the bound at the lists' last entries
+    (3, 20, 20, 0),        # one split, every token listed
+    (4, 40000, 16, 2),     # two rows of equal logits: every list entry is a candidate
+])
+def test_lmhead_merge_lists(n, V, k, zero):
+    h, w = synth.lmhead_inputs(17, n, V, 64)
+    h[:zero] = 0
+    check(h, w, k, rows=np.unique(np.linspace(0, n - 1, 40).astype(int)))
+
+
 @pytest.mark.parametrize("n,d,V,k", [
     (200, 128, 1000, 10),     # ragged rows and vocabulary, one tile per CTA
     (64, 64, 151936, 1),      # one K slice; the last vocabulary tile holds 128 tokens
