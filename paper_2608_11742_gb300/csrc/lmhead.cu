@@ -7,24 +7,31 @@
 // statistics are folded in its epilogue, so the logits never reach HBM.
 //
 // Contraction. A CTA owns one tile of 128 hidden rows and one contiguous range
-// of 256-token vocabulary tiles (a "split"); the CTAs of every row tile take
-// the same splits, so they stream the same unembedding tiles at the same pace
-// and each tile comes from HBM once, the other row tiles finding it in L2.
-//   warp 0      TMA producer: per 64-wide slice of d, the hidden tile (128 x
-//               64) and the unembedding tile (256 x 64), 128-byte swizzle,
-//               into a ring of kStages shared-memory stages (mbarrier
-//               completion, bounded waits);
-//   warp 1      MMA issuer: tcgen05.mma kind::f16 (bf16 x bf16 -> f32), M = 128,
-//               N = 256, K = 16, four per stage, into one of two TMEM
-//               accumulators (128 lanes x 256 columns each), so that the
-//               epilogue of one tile overlaps the contraction of the next;
-//               it also allocates and frees the 512 TMEM columns;
+// of the vocabulary (a "split"), walked in tiles of 256 tokens; the CTAs of
+// every row tile take the same splits, so they stream the same unembedding
+// tiles at the same pace and each tile comes from HBM once, the other row tiles
+// finding it in L2. Two row tiles can share a CTA pair (cta_group::2): M = 256
+// over both, half of each unembedding tile in either CTA.
+//   warp 0      TMA producer: per stage, the hidden tile's and the unembedding
+//               tile's 64-wide slices of d, 128-byte swizzle, into a ring of
+//               shared-memory stages (mbarrier completion, bounded waits). A
+//               pair takes two slices per stage and one copy per operand: with
+//               a copy per 64 rows and slice the one issuing thread set the pace
+//               (512 rows: 329 us against 309);
+//   warp 1      MMA issuer (the pair's first CTA): tcgen05.mma kind::f16 (bf16 x
+//               bf16 -> f32), M = 128 or 256, N = 256, K = 16, four per slice,
+//               into one of two TMEM accumulators (128 lanes x 256 columns each),
+//               so that the epilogue of one tile overlaps the contraction of the
+//               next; it also allocates and frees the 512 TMEM columns;
 //   warps 2-5   epilogue: thread = row (TMEM lane). tcgen05.ld brings its 256
 //               logits; pass 1 finds the tile maximum, pass 2 folds the
 //               logits into the row's base-2 online softmax record (B, S, T
 //               with S = sum 2^u, T = sum u 2^u, u = z log2(e) - B), the
 //               running maximum and argmax, and, in top-k mode, a sorted
-//               register list of the KMAX largest logits.
+//               register list of the KMAX largest logits. A warp inserts as
+//               often as its busiest lane, so few columns may enter: the first
+//               tile's group maxima bound the k-th logit before any does (200
+//               rows, V 32,000, d 1,024, k 10: 72 -> 36 us with the pairs).
 // At the end of its range each epilogue thread leaves its row's record and
 // list in the workspace; a second launch (one warp per row) merges the splits
 // and writes the statistics, with the same formulas as the streaming kernel.
@@ -54,15 +61,26 @@ constexpr int kTileM = 128;                 // hidden rows per tile (TMEM lanes)
 constexpr int kTileN = 256;                 // tokens per tile (accumulator columns)
 constexpr int kTileK = 64;                  // d per stage: one 128-byte swizzle row of bf16
 constexpr int kMmaK = 16;                   // K of one tcgen05.mma kind::f16
-constexpr int kStages = 4;
 constexpr int kABytes = kTileM * kTileK * 2;  // 16 KB
 constexpr int kBBytes = kTileN * kTileK * 2;  // 32 KB
-constexpr int kStageBytes = kABytes + kBBytes;
-constexpr int kThreads = 192;               // warp 0 TMA, warp 1 MMA, warps 2-5 epilogue
 constexpr int kEpiWarps = 4;
+constexpr int kMaxStages = 4;
+constexpr int kLineRows = 16;               // packed rows (128 bytes each) per line of the pair's tensor map
+// Shape of the contraction by CTA group: one CTA (CG 1) with the whole
+// unembedding tile in its stages, or a pair (CG 2) with half of it each.
+template <int CG>
+struct Shape {
+    static constexpr int stages = CG == 1 ? 4 : 3;
+    static constexpr int slices = CG == 1 ? 1 : 2;              // 64-wide slices of d per stage
+    static constexpr int stage_bytes = slices * (kABytes + kBBytes / CG);
+    // the ring, 32 logits per epilogue thread, and slack to align the ring to 1024 bytes
+    static constexpr int smem_bytes = stages * stage_bytes + kEpiWarps * 32 * 32 * 4 + 1024;
+    static constexpr int granule = CG == 1 ? kTileN : kTileN / 2;   // tokens the splits are cut at
+    static_assert(stages <= kMaxStages, "");
+};
+constexpr int kThreads = 192;               // warp 0 TMA, warp 1 MMA, warps 2-5 epilogue
 constexpr uint32_t kTmemCols = 2 * kTileN;  // two accumulators
 constexpr int kMaxSplits = 256;
-constexpr int kSmemBytes = kStages * kStageBytes + 1024;  // + slack to align the ring to 1024 bytes
 constexpr int kMergeThreads = 128;
 constexpr uint64_t kDrainNs = 200ull * 1000 * 1000;
 constexpr float kLog2e = 1.4426950408889634f;
@@ -79,7 +97,7 @@ struct __align__(16) LmPartial {
 };
 
 struct LmArgs {
-    int32_t n_rows, d, n_vt, splits, kmax, k;
+    int32_t n_rows, d, n_gran, splits, kmax, k;  // n_gran: granules of the vocabulary
     const uint8_t *w_packed;  // unembedding in the packed tile layout, or nullptr (tensor map)
     int64_t vocab;
     LmPartial *part;   // [n_rows][splits]
@@ -104,11 +122,12 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
 __device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(saddr(bar)), "r"(bytes) : "memory");
 }
+// (cluster scope: the arrival may come from the pair's other CTA)
 __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
     uint32_t done;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(done)
         : "r"(saddr(bar)), "r"(parity)
@@ -128,6 +147,32 @@ __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, i
         "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(saddr(bar))
         : "memory");
 }
+// The same as half of a CTA pair: `bar` is a cluster address, in either CTA of the pair.
+__device__ __forceinline__ void tma_load_3d_pair(void *dst, const CUtensorMap *map, int c0, int c1, int c2,
+                                                 uint32_t bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, "
+        "%3, %4}], [%5];" ::"r"(saddr(dst)),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(bar)
+        : "memory");
+}
+// Cluster address of `p`'s counterpart in CTA 0 of the cluster.
+__device__ __forceinline__ uint32_t leader_addr(const void *p) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(saddr(p)));
+    return r;
+}
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
 // Plain bulk copy of `bytes` contiguous bytes into shared memory, completing on `bar`.
 __device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t bytes, uint64_t *bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
@@ -139,33 +184,64 @@ __device__ __forceinline__ void prefetch_map(const CUtensorMap *map) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
 }
 
+template <int CG>
 __device__ __forceinline__ void tmem_alloc(uint32_t *slot, uint32_t ncols) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(saddr(slot)), "r"(ncols)
-                 : "memory");
+    if constexpr (CG == 1)
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(saddr(slot)), "r"(ncols)
+                     : "memory");
+    else
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(saddr(slot)), "r"(ncols)
+                     : "memory");
 }
+template <int CG>
 __device__ __forceinline__ void tmem_relinquish() {
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    if constexpr (CG == 1) asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    else asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
 }
+template <int CG>
 __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
+    if constexpr (CG == 1)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
+    else
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// D[tmem] (+)= A[smem] x B[smem]^T, bf16 inputs, f32 accumulator; accumulate != 0 adds to D.
+// D[tmem] (+)= A[smem] x B[smem]^T, bf16 inputs, f32 accumulator; accumulate != 0
+// adds to D. CG 2: A, B and D are spread over the pair, half in each CTA at the
+// same addresses.
+template <int CG>
 __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
                                          uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
+    if constexpr (CG == 1)
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "setp.ne.b32 p, %4, 0;\n\t"
+            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+            "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+            : "memory");
+    else
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "setp.ne.b32 p, %4, 0;\n\t"
+            "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+            "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+            : "memory");
 }
-// Arrives on `bar` once every tcgen05 operation this thread issued before has completed.
+// Arrives on `bar` once every tcgen05 operation this thread issued before has
+// completed; CG 2: on the barrier's counterpart in both CTAs of the pair.
+template <int CG>
 __device__ __forceinline__ void mma_commit(uint64_t *bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(saddr(bar))
-                 : "memory");
+    if constexpr (CG == 1)
+        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(saddr(bar))
+                     : "memory");
+    else
+        asm volatile(
+            "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+                saddr(bar)),
+            "h"(static_cast<uint16_t>(3))
+            : "memory");
 }
 
 // 32 consecutive f32 columns of this thread's TMEM lane (the warp's 32 lanes at once).
@@ -193,7 +269,7 @@ __device__ __forceinline__ float ex2(float x) {
 
 // ---------------------------------------------------------------- bounded waits
 struct Ctl {
-    uint64_t full[kStages], empty[kStages], acc_full[2], acc_empty[2], mma_done;
+    uint64_t full[kMaxStages], empty[kMaxStages], acc_full[2], acc_empty[2], mma_done;
     uint32_t tmem_base;
     int abort_flag;
     int skip;
@@ -242,32 +318,49 @@ struct RowState {
 
 // Inserts (z, id) into the sorted list (logit desc; ids arrive in increasing
 // order, so equal logits keep the lower id first). Called for z > lv[KMAX-1].
+// Every entry is formed from the old list (itself, its neighbour or z), so the
+// steps do not wait for one another.
 template <int KMAX>
 __device__ __forceinline__ void list_insert(RowState<KMAX> &st, float z, int id) {
-    float cv = z;
-    int ci = id;
 #pragma unroll
-    for (int i = 0; i < KMAX; ++i) {
-        const bool sw = cv > st.lv[i];
-        const float tv = st.lv[i];
-        const int ti = st.li[i];
-        st.lv[i] = sw ? cv : tv;
-        st.li[i] = sw ? ci : ti;
-        cv = sw ? tv : cv;
-        ci = sw ? ti : ci;
+    for (int i = KMAX - 1; i > 0; --i) {
+        const float cur = st.lv[i], up = st.lv[i - 1];
+        const int cur_i = st.li[i], up_i = st.li[i - 1];
+        const float v = z > up ? up : z;
+        const int vi = z > up ? up_i : id;
+        st.lv[i] = z > cur ? v : cur;
+        st.li[i] = z > cur ? vi : cur_i;
     }
+    const float top = st.lv[0];
+    const int top_i = st.li[0];
+    st.lv[0] = z > top ? z : top;
+    st.li[0] = z > top ? id : top_i;
 }
 
-template <int KMAX>
+// The float below x (-inf and NaN stay).
+__device__ __forceinline__ float next_below(float x) {
+    if (!(x > -INFINITY)) return x;
+    if (x == 0.f) return __uint_as_float(0x80000001u);
+    const uint32_t b = __float_as_uint(x);
+    return __uint_as_float(x > 0.f ? b - 1 : b + 1);
+}
+
+template <int KMAX, int CG>
 __global__ void __launch_bounds__(kThreads, 1)
-    lmhead_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_constant__ CUtensorMap tm_w, const LmArgs a) {
+    lmhead_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_constant__ CUtensorMap tm_w,
+                  const __grid_constant__ CUtensorMap tm_w_half, const LmArgs a) {
+    using Sh = Shape<CG>;
+    constexpr int kStages = Sh::stages;
+    constexpr int kStageBytes = Sh::stage_bytes;
     extern __shared__ uint8_t dyn_smem[];
     __shared__ Ctl c;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int rt = blockIdx.x / a.splits, split = blockIdx.x - rt * a.splits;
-    const int vt0 = static_cast<int>(static_cast<int64_t>(split) * a.n_vt / a.splits);
-    const int vt1 = static_cast<int>(static_cast<int64_t>(split + 1) * a.n_vt / a.splits);
-    const int n_tiles = vt1 - vt0;
+    const int rank = CG == 1 ? 0 : static_cast<int>(cluster_rank());
+    const int unit = static_cast<int>(blockIdx.x) / CG;  // CTA or pair
+    const int rt = unit / a.splits * CG + rank, split = unit % a.splits;
+    const int col_begin = static_cast<int>(static_cast<int64_t>(split) * a.n_gran / a.splits) * Sh::granule;
+    const int col_end = static_cast<int>(static_cast<int64_t>(split + 1) * a.n_gran / a.splits) * Sh::granule;
+    const int n_tiles = (col_end - col_begin + kTileN - 1) / kTileN;
     const int kblocks = a.d / kTileK;
     // the ring starts on a 1024-byte boundary (the 128-byte swizzle's period)
     uint8_t *ring = dyn_smem + ((1024u - (saddr(dyn_smem) & 1023u)) & 1023u);
@@ -279,7 +372,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&c.acc_full[b], 1);
-            mbar_init(&c.acc_empty[b], kEpiWarps);
+            mbar_init(&c.acc_empty[b], kEpiWarps * CG);
         }
         mbar_init(&c.mma_done, 1);
         c.abort_flag = 0;
@@ -290,8 +383,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         prefetch_map(&tm_w);
     }
     if (warp == 1) {
-        tmem_alloc(&c.tmem_base, kTmemCols);
-        tmem_relinquish();
+        tmem_alloc<CG>(&c.tmem_base, kTmemCols);
+        tmem_relinquish<CG>();
     }
     // the hidden rows may come from the previous kernel on the stream
     pdl_wait();
@@ -299,6 +392,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (threadIdx.x == 0) c.skip = __ldcg(a.health) != 0;
     tc_fence_before();
     __syncthreads();
+    if constexpr (CG == 2) {
+        cluster_sync();  // the pair's barriers are initialised
+        __syncwarp();
+    }
     tc_fence_after();
     const uint32_t tmem = c.tmem_base;
     if (c.skip) {  // a workspace an earlier launch gave up on: write nothing
@@ -308,8 +405,9 @@ __global__ void __launch_bounds__(kThreads, 1)
             uint32_t it = 0;
             bool ok = true;
             for (int t = 0; t < n_tiles && ok; ++t) {
-                const int vt = vt0 + t;
-                for (int kb = 0; kb < kblocks; ++kb) {
+                const int col0 = col_begin + t * kTileN;
+                const int n_cols = min(kTileN, col_end - col0);  // CG 2: 256, or 128 in a range's last tile
+                for (int kb = 0; kb < kblocks; kb += Sh::slices) {
                     const int s = it % kStages;
                     const uint32_t ph = (it / kStages) & 1;
                     if (!wait_or_abort(&c.empty[s], ph ^ 1, c, a)) {
@@ -317,24 +415,44 @@ __global__ void __launch_bounds__(kThreads, 1)
                         break;
                     }
                     uint8_t *sa = ring + s * kStageBytes;
-                    mbar_expect_tx(&c.full[s], kStageBytes);
-                    tma_load_2d(sa, &tm_h, kb * kTileK, rt * kTileM, &c.full[s]);
-                    if (a.w_packed)  // one contiguous 32 KB block, already in the swizzled image
-                        bulk_load(sa + kABytes, a.w_packed + (static_cast<int64_t>(vt) * kblocks + kb) * kBBytes,
-                                  kBBytes, &c.full[s]);
-                    else
-                        tma_load_2d(sa + kABytes, &tm_w, kb * kTileK, vt * kTileN, &c.full[s]);
+                    if constexpr (CG == 1) {
+                        mbar_expect_tx(&c.full[s], kStageBytes);
+                        tma_load_2d(sa, &tm_h, kb * kTileK, rt * kTileM, &c.full[s]);
+                        if (a.w_packed)  // one contiguous 32 KB block, already in the swizzled image
+                            bulk_load(sa + kABytes,
+                                      a.w_packed + (static_cast<int64_t>(col0 / kTileN) * kblocks + kb) * kBBytes, kBBytes,
+                                      &c.full[s]);
+                        else
+                            tma_load_2d(sa + kABytes, &tm_w, kb * kTileK, col0, &c.full[s]);
+                    } else {
+                        // both CTAs' copies complete on the leader's barrier, which
+                        // expects the bytes of both
+                        const uint32_t bar = leader_addr(&c.full[s]);
+                        if (rank == 0)
+                            mbar_expect_tx(&c.full[s], Sh::slices * (2 * kABytes + n_cols * kTileK * 2));
+                        // one copy per operand for all slices of the stage (past the last
+                        // slice of d it brings values that no MMA reads)
+                        tma_load_3d_pair(sa, &tm_h, 0, rt * kTileM, kb, bar);
+                        const int tok = col0 + rank * (n_cols / 2);  // this CTA's half of the tile's tokens
+                        const CUtensorMap *map = n_cols == kTileN ? &tm_w : &tm_w_half;
+                        uint8_t *sb = sa + Sh::slices * kABytes;
+                        // packed: 16 rows of the swizzled image per 2 KB line of the map
+                        if (a.w_packed)
+                            tma_load_3d_pair(sb, map, 0, tok % kTileN / kLineRows, tok / kTileN * kblocks + kb, bar);
+                        else
+                            tma_load_3d_pair(sb, map, 0, tok, kb, bar);
+                    }
                     ++it;
                 }
             }
             // every copy issued lands before the CTA leaves, whichever role
-            // aborted (in a normal run these phases have long completed)
+            // aborted (in a normal run these phases have long completed). The
+            // second CTA of a pair sees it by its stages being consumed.
             for (uint32_t j = it > kStages ? it - kStages : 0; j < it; ++j)
-                wait_drain(&c.full[j % kStages], (j / kStages) & 1);
+                wait_drain(rank == 0 ? &c.full[j % kStages] : &c.empty[j % kStages], (j / kStages) & 1);
         }
     } else if (warp == 1) {
-        if (lane == 0) {  // ---------------------------------------- MMA issuer
-            constexpr uint32_t idesc = umma::instr_desc_bf16(kTileM, kTileN);
+        if (lane == 0 && rank == 0) {  // --------------------------- MMA issuer
             uint32_t it = 0;
             bool ok = true;
             for (int t = 0; t < n_tiles && ok; ++t) {
@@ -343,7 +461,9 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (!wait_or_abort(&c.acc_empty[buf], (use & 1) ^ 1, c, a)) break;
                 tc_fence_after();
                 const uint32_t d_tmem = tmem + static_cast<uint32_t>(buf * kTileN);
-                for (int kb = 0; kb < kblocks; ++kb) {
+                const int n_cols = min(kTileN, col_end - (col_begin + t * kTileN));
+                const uint32_t idesc = umma::instr_desc_bf16(kTileM * CG, n_cols);
+                for (int kb = 0; kb < kblocks; kb += Sh::slices) {
                     const int s = it % kStages;
                     const uint32_t ph = (it / kStages) & 1;
                     if (!wait_or_abort(&c.full[s], ph, c, a)) {
@@ -351,20 +471,26 @@ __global__ void __launch_bounds__(kThreads, 1)
                         break;
                     }
                     tc_fence_after();
-                    const uint32_t sa = saddr(ring + s * kStageBytes);
-                    const uint64_t ad = umma::smem_desc_kmajor_sw128(sa);
-                    const uint64_t bd = umma::smem_desc_kmajor_sw128(sa + kABytes);
 #pragma unroll
-                    for (int k = 0; k < kTileK / kMmaK; ++k)
-                        mma_bf16(d_tmem, umma::advance_k16(ad, k), umma::advance_k16(bd, k), idesc,
-                                 (kb | k) != 0 ? 1u : 0u);
-                    mma_commit(&c.empty[s]);  // the stage is free once these MMAs have read it
+                    for (int j = 0; j < Sh::slices; ++j) {
+                        if (j > 0 && kb + j >= kblocks) break;
+                        const uint32_t sa = saddr(ring + s * kStageBytes);
+                        const uint64_t ad = umma::smem_desc_kmajor_sw128(sa + j * kABytes);
+                        const uint64_t bd =
+                            umma::smem_desc_kmajor_sw128(sa + Sh::slices * kABytes + j * (n_cols / CG * kTileK * 2));
+#pragma unroll
+                        for (int k = 0; k < kTileK / kMmaK; ++k) {
+                            mma_bf16<CG>(d_tmem, umma::advance_k16(ad, k), umma::advance_k16(bd, k), idesc,
+                                         (kb | j | k) != 0 ? 1u : 0u);
+                        }
+                    }
+                    mma_commit<CG>(&c.empty[s]);  // the stage is free once these MMAs have read it
                     ++it;
                 }
-                if (ok) mma_commit(&c.acc_full[buf]);
+                if (ok) mma_commit<CG>(&c.acc_full[buf]);
             }
             // every MMA issued has completed before TMEM is freed
-            mma_commit(&c.mma_done);
+            mma_commit<CG>(&c.mma_done);
             wait_drain(&c.mma_done, 0);
         }
         __syncwarp();
@@ -383,6 +509,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             st.lv[i] = -INFINITY;
             st.li[i] = INT_MAX;
         }
+        float floor_thr = -INFINITY;  // logits up to this never enter the list
+        float *pick = reinterpret_cast<float *>(ring + kStages * kStageBytes) + (warp - 2) * 32 + lane;
         bool ok = true;
         for (int t = 0; t < n_tiles; ++t) {
             const int buf = t & 1;
@@ -393,12 +521,17 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
             tc_fence_after();
             const uint32_t tbase = tmem + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(buf * kTileN);
-            const int col0 = (vt0 + t) * kTileN;
-            const int ncol = static_cast<int>(min(static_cast<int64_t>(kTileN), a.vocab - col0));
-            // pass 1: the tile's maximum and its lowest column
+            const int col0 = col_begin + t * kTileN;
+            const int ncol = static_cast<int>(min(static_cast<int64_t>(min(kTileN, col_end - col0)), a.vocab - col0));
+            const int n_ch = (ncol + 31) / 32;
+            // pass 1: the tile's maximum and its lowest column. In the first tile
+            // of a list, the maxima of its groups of columns bound the row's k-th
+            // logit from below (k groups each hold one at least that large), so
+            // that few columns enter the list (see pass 2).
+            constexpr int kGroup = KMAX > 16 ? 8 : 16;  // at least KMAX groups in a whole tile
             float tm = -INFINITY;
             int ta = INT_MAX;
-            for (int ch = 0; ch < kTileN / 32; ++ch) {
+            for (int ch = 0; ch < n_ch; ++ch) {
                 float v[32];
                 tmem_ld32(tbase + ch * 32, v);
 #pragma unroll
@@ -409,6 +542,26 @@ __global__ void __launch_bounds__(kThreads, 1)
                         ta = col0 + cc;
                     }
                 }
+                if (KMAX > 0 && t == 0) {
+#pragma unroll 1
+                    for (int g = 0; g < 32; g += kGroup) {
+                        float gm = -INFINITY;
+#pragma unroll
+                        for (int i = 0; i < 32; ++i)
+                            if (i / kGroup * kGroup == g && ch * 32 + i < ncol) gm = fmaxf(gm, v[i]);
+                        list_insert<KMAX>(st, gm, INT_MAX);
+                    }
+                }
+            }
+            if (KMAX > 0 && t == 0) {
+                float kth = -INFINITY;
+#pragma unroll
+                for (int i = 0; i < (KMAX > 0 ? KMAX : 1); ++i) {
+                    kth = fmaxf(kth, i >= a.k - 1 ? st.lv[i] : -INFINITY);  // (sorted: entry k - 1)
+                    st.lv[i] = -INFINITY;
+                    st.li[i] = INT_MAX;
+                }
+                floor_thr = next_below(kth);
             }
             if (tm > st.mx) {
                 st.mx = tm;
@@ -426,7 +579,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 st.B = nb;
             }
             // pass 2: the sums, the top-k list, and (testing only) the logits
-            for (int ch = 0; ch < kTileN / 32; ++ch) {
+            for (int ch = 0; ch < n_ch; ++ch) {
                 float v[32];
                 tmem_ld32(tbase + ch * 32, v);
                 const int nv = min(32, ncol - ch * 32);  // valid columns of this chunk (32 but in the last tile)
@@ -437,7 +590,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
                 float ps[2] = {0.f, 0.f}, pt[2] = {0.f, 0.f};
                 uint32_t cand = 0;  // columns that pass the list's last entry
-                const float thr = KMAX > 0 ? st.lv[KMAX > 0 ? KMAX - 1 : 0] : INFINITY;
+                const float thr = KMAX > 0 ? fmaxf(st.lv[KMAX > 0 ? KMAX - 1 : 0], floor_thr) : INFINITY;
 #pragma unroll
                 for (int i = 0; i < 32; ++i) {
                     const float u = fmaf(v[i], kLog2e, -st.B);
@@ -449,15 +602,19 @@ __global__ void __launch_bounds__(kThreads, 1)
                 st.s += ps[0] + ps[1];
                 st.t += pt[0] + pt[1];
                 // the few candidates, one copy of the insertion (the list only
-                // grows stricter, so each is checked again against it)
-#pragma unroll 1
-                while (KMAX > 0 && cand) {
-                    const int i = __ffs(cand) - 1;
-                    cand &= cand - 1;
-                    float x = v[0];
+                // grows stricter, so each is checked again against it), their
+                // logits picked by index from shared memory
+                if (KMAX > 0 && __any_sync(kFull, cand != 0)) {
 #pragma unroll
-                    for (int j = 1; j < 32; ++j) x = j == i ? v[j] : x;
-                    if (x > st.lv[KMAX > 0 ? KMAX - 1 : 0]) list_insert<KMAX>(st, x, col0 + ch * 32 + i);
+                    for (int i = 0; i < 32; ++i) pick[i * (kEpiWarps * 32)] = v[i];
+#pragma unroll 1
+                    while (cand) {
+                        const int i = __ffs(cand) - 1;
+                        cand &= cand - 1;
+                        const float x = pick[i * (kEpiWarps * 32)];
+                        if (x > st.lv[KMAX > 0 ? KMAX - 1 : 0]) list_insert<KMAX>(st, x, col0 + ch * 32 + i);
+                    }
+                    __syncwarp();
                 }
                 if (a.logits_out && live) {
                     float *dst = a.logits_out + static_cast<int64_t>(row) * a.vocab + col0 + ch * 32;
@@ -467,7 +624,10 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&c.acc_empty[buf]);
+            if (lane == 0) {
+                if constexpr (CG == 1) mbar_arrive(&c.acc_empty[buf]);
+                else mbar_arrive_cluster(leader_addr(&c.acc_empty[buf]));
+            }
         }
         if (ok && live) {
             const int64_t slot = static_cast<int64_t>(row) * a.splits + split;
@@ -488,8 +648,16 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     tc_fence_before();
     __syncthreads();
+    if constexpr (CG == 2) {
+        // neither CTA leaves while the other's copies, MMAs or arrivals may reach
+        // it: the last commit arrives in both
+        if (rank != 0 && threadIdx.x == 0 && !c.skip) wait_drain(&c.mma_done, 0);
+        __syncwarp();
+        cluster_sync();
+        __syncwarp();
+    }
     tc_fence_after();
-    if (warp == 1) tmem_dealloc(tmem, kTmemCols);
+    if (warp == 1) tmem_dealloc<CG>(tmem, kTmemCols);
 }
 
 // ---------------------------------------------------------------- merge
@@ -700,7 +868,65 @@ __global__ void pack_unembed_kernel(const uint4 *w, int64_t vocab, int32_t d, in
 struct LmDevice {
     bool ready = false;
     int sm_count = 0;
+    int pairs = 0;  // CTA pairs resident at once
 };
+
+// Tensor maps of one launch: hidden rows, unembedding tiles, half tiles (pairs).
+struct LmMaps {
+    CUtensorMap h, w, w_half;
+};
+
+template <int CG>
+void lm_config(cudaLaunchConfig_t *cfg, cudaLaunchAttribute (&attr)[2], dim3 grid, cudaStream_t stream) {
+    *cfg = cudaLaunchConfig_t{};
+    cfg->gridDim = grid;
+    cfg->blockDim = dim3(kThreads);
+    cfg->dynamicSmemBytes = Shape<CG>::smem_bytes;
+    cfg->stream = stream;
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = CG;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cfg->attrs = attr;
+    cfg->numAttrs = CG == 1 ? 1 : 2;
+}
+
+template <int KMAX, int CG>
+cudaError_t launch_lm(int grid, cudaStream_t stream, const LmMaps &m, const LmArgs &a) {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[2];
+    lm_config<CG>(&cfg, attr, dim3(grid), stream);
+    return cudaLaunchKernelEx(&cfg, lmhead_kernel<KMAX, CG>, m.h, m.w, m.w_half, a);
+}
+
+template <int CG>
+cudaError_t launch_lm_k(int grid, cudaStream_t stream, const LmMaps &m, const LmArgs &a) {
+    return a.kmax == 0    ? launch_lm<0, CG>(grid, stream, m, a)
+           : a.kmax == 12 ? launch_lm<12, CG>(grid, stream, m, a)
+           : a.kmax == 16 ? launch_lm<16, CG>(grid, stream, m, a)
+                          : launch_lm<32, CG>(grid, stream, m, a);
+}
+
+template <int KMAX>
+cudaError_t set_smem() {
+    cudaError_t e = cudaFuncSetAttribute(lmhead_kernel<KMAX, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         Shape<1>::smem_bytes);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(lmhead_kernel<KMAX, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 Shape<2>::smem_bytes);
+    return e;
+}
+
+// Resident CTA pairs of the widest form (the others need no more).
+cudaError_t count_pairs(int *pairs) {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[2];
+    lm_config<2>(&cfg, attr, dim3(2), nullptr);
+    cfg.attrs = attr + 1;
+    cfg.numAttrs = 1;
+    return cudaOccupancyMaxActiveClusters(pairs, lmhead_kernel<32, 2>, &cfg);
+}
 constexpr int kMaxDevices = 64;
 std::mutex g_lm_mutex;
 LmDevice g_lm_devices[kMaxDevices];
@@ -722,20 +948,23 @@ rps_status lm_device(LmDevice *out) {
     LmDevice &d = g_lm_devices[dev];
     if (!d.ready) {
         if (cudaDeviceGetAttribute(&d.sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return RPS_ERR_CUDA;
-        const int kmaxes[3] = {0, 16, 32};
-        for (int i = 0; i < 3; ++i) {
-            cudaError_t e = kmaxes[i] == 0   ? cudaFuncSetAttribute(lmhead_kernel<0>,
-                                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes)
-                            : kmaxes[i] == 16 ? cudaFuncSetAttribute(lmhead_kernel<16>,
-                                                                     cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes)
-                                              : cudaFuncSetAttribute(lmhead_kernel<32>,
-                                                                     cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-            if (e != cudaSuccess) return RPS_ERR_CUDA;
-        }
+        if (set_smem<0>() != cudaSuccess || set_smem<12>() != cudaSuccess || set_smem<16>() != cudaSuccess || set_smem<32>() != cudaSuccess)
+            return RPS_ERR_CUDA;
+        if (count_pairs(&d.pairs) != cudaSuccess) return RPS_ERR_CUDA;
         d.ready = true;
     }
     *out = d;
     return RPS_OK;
+}
+
+rps_status encode(CUtensorMap *m, CUtensorMapDataType type, int rank, const void *base, const cuuint64_t *dims,
+                  const cuuint64_t *strides, const cuuint32_t *box, bool swizzle) {
+    const cuuint32_t es[3] = {1, 1, 1};
+    const CUresult r = g_encode(m, type, rank, const_cast<void *>(base), dims, strides, box, es,
+                                CU_TENSOR_MAP_INTERLEAVE_NONE,
+                                swizzle ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
+                                CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? RPS_OK : RPS_ERR_CUDA;
 }
 
 // 2-D bf16 tensor map over rows x d (d contiguous), box of 64 x box_rows, 128-byte swizzle.
@@ -743,14 +972,29 @@ rps_status make_map(CUtensorMap *m, const void *base, int64_t rows, int32_t d, i
     const cuuint64_t dims[2] = {static_cast<cuuint64_t>(d), static_cast<cuuint64_t>(rows)};
     const cuuint64_t strides[1] = {static_cast<cuuint64_t>(stride_elems) * 2};
     const cuuint32_t box[2] = {static_cast<cuuint32_t>(kTileK), static_cast<cuuint32_t>(box_rows)};
-    const cuuint32_t es[2] = {1, 1};
-    const CUresult r = g_encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), dims, strides, box, es,
-                                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                                CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS ? RPS_OK : RPS_ERR_CUDA;
+    return encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base, dims, strides, box, true);
 }
 
-int list_len(int32_t k) { return k == 0 ? 0 : (k <= 16 ? 16 : 32); }
+// The same rows x d as 64 x rows x (d / 64): a box holds `box_rows` rows of a
+// stage's slices, slice after slice, 128-byte swizzle.
+rps_status make_slice_map(CUtensorMap *m, const void *base, int64_t rows, int32_t d, int64_t stride_elems,
+                          int box_rows) {
+    const cuuint64_t dims[3] = {kTileK, static_cast<cuuint64_t>(rows), static_cast<cuuint64_t>(d / kTileK)};
+    const cuuint64_t strides[2] = {static_cast<cuuint64_t>(stride_elems) * 2, kTileK * 2};
+    const cuuint32_t box[3] = {kTileK, static_cast<cuuint32_t>(box_rows), Shape<2>::slices};
+    return encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, base, dims, strides, box, true);
+}
+
+// The packed unembedding as 2 KB lines (16 of its 128-byte rows, 256 64-bit
+// words) x 16 lines x blocks, no swizzle (the blocks hold the swizzled image).
+rps_status make_packed_map(CUtensorMap *m, const void *base, int64_t blocks, int box_rows) {
+    const cuuint64_t dims[3] = {256, kTileN / kLineRows, static_cast<cuuint64_t>(blocks)};
+    const cuuint64_t strides[2] = {2048, kBBytes};
+    const cuuint32_t box[3] = {256, static_cast<cuuint32_t>(box_rows / kLineRows), Shape<2>::slices};
+    return encode(m, CU_TENSOR_MAP_DATA_TYPE_INT64, 3, base, dims, strides, box, false);
+}
+
+int list_len(int32_t k) { return k == 0 ? 0 : k <= 12 ? 12 : k <= 16 ? 16 : 32; }
 
 struct LmLayout {
     size_t health, part, lists, total;
@@ -825,20 +1069,42 @@ rps_status rps_lmhead_row_stats(const rps_lmhead *lm, const rps_params *prm, con
 
     const int n_rt = (lm->n_rows + kTileM - 1) / kTileM;
     const int n_vt = static_cast<int>((lm->vocab + kTileN - 1) / kTileN);
-    const int splits = std::max(1, std::min({dev.sm_count / n_rt, n_vt, kMaxSplits}));
-    CUtensorMap tm_h, tm_w;
-    if ((st = make_map(&tm_h, lm->hidden, lm->n_rows, lm->d, lm->hidden_stride, kTileM)) != RPS_OK) return st;
-    if (lm->unembed_packed) {  // the tensor map is not read; the hidden map stands in its slot
-        tm_w = tm_h;
-    } else if ((st = make_map(&tm_w, lm->unembed, lm->vocab, lm->d, lm->unembed_stride, kTileN)) != RPS_OK) {
-        return st;
+    // CTA pairs or single CTAs. A pair shares each unembedding tile, half in each
+    // CTA: 32 KB per 64-wide slice and CTA instead of 48, from L2 and into shared
+    // memory. An odd row tile makes a pair with an empty half, which costs as much
+    // as two tiles: at 3 and 5 row tiles that is more than the pairs save. One row
+    // tile alone is bound by reading the unembedding. V 126,464, d 4,096, statistics
+    // only, single against pairs: 200 rows 232 / 189 us, 300 rows 271 / 292, 512 rows
+    // 338 / 309, 640 rows 442 / 447, 896 rows 605 / 586, 1,152 rows 765 / 734.
+    // (The packed unembedding's blocks are tensor coordinates in a pair, 32 bits.)
+    const int kblocks = lm->d / kTileK;
+    const int64_t packed_blocks = static_cast<int64_t>(n_vt) * kblocks;
+    const bool pair = (n_rt % 2 == 0 || n_rt >= 7) && dev.pairs >= 1 && packed_blocks <= INT32_MAX;
+    const int units = pair ? (n_rt + 1) / 2 : n_rt;  // pairs or CTAs per split
+    const int splits = std::max(1, std::min({(pair ? dev.pairs : dev.sm_count) / units, n_vt, kMaxSplits}));
+    LmMaps maps;
+    std::memset(&maps, 0, sizeof maps);
+    if (pair) {
+        st = make_slice_map(&maps.h, lm->hidden, lm->n_rows, lm->d, lm->hidden_stride, kTileM);
+        for (int half = 0; half < 2 && st == RPS_OK; ++half) {
+            CUtensorMap *m = half ? &maps.w_half : &maps.w;
+            const int rows = kTileN / 2 >> half;  // one CTA's tokens
+            st = lm->unembed_packed ? make_packed_map(m, lm->unembed, packed_blocks, rows)
+                                    : make_slice_map(m, lm->unembed, lm->vocab, lm->d, lm->unembed_stride, rows);
+        }
+        if (st != RPS_OK) return st;
+    } else {
+        if ((st = make_map(&maps.h, lm->hidden, lm->n_rows, lm->d, lm->hidden_stride, kTileM)) != RPS_OK) return st;
+        maps.w = maps.h;  // (single CTAs read the packed unembedding without a tensor map)
+        if (!lm->unembed_packed &&
+            (st = make_map(&maps.w, lm->unembed, lm->vocab, lm->d, lm->unembed_stride, kTileN)) != RPS_OK)
+            return st;
     }
 
     LmArgs a;
     std::memset(&a, 0, sizeof a);
     a.n_rows = lm->n_rows;
     a.d = lm->d;
-    a.n_vt = n_vt;
     a.splits = splits;
     a.kmax = list_len(k);
     a.k = k;
@@ -862,14 +1128,13 @@ rps_status rps_lmhead_row_stats(const rps_lmhead *lm, const rps_params *prm, con
     a.topk_logit = out->topk_logit;
 
     const cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    const dim3 grid(n_rt * splits), block(kThreads);
-    cudaError_t e;
-    if (a.kmax == 0) e = launch_pdl(lmhead_kernel<0>, grid, block, kSmemBytes, s, tm_h, tm_w, a);
-    else if (a.kmax == 16) e = launch_pdl(lmhead_kernel<16>, grid, block, kSmemBytes, s, tm_h, tm_w, a);
-    else e = launch_pdl(lmhead_kernel<32>, grid, block, kSmemBytes, s, tm_h, tm_w, a);
+    const int granule = pair ? Shape<2>::granule : Shape<1>::granule;
+    a.n_gran = static_cast<int>((lm->vocab + granule - 1) / granule);
+    cudaError_t e = pair ? launch_lm_k<2>(units * splits * 2, s, maps, a) : launch_lm_k<1>(units * splits, s, maps, a);
     if (e != cudaSuccess) return RPS_ERR_CUDA;
     const dim3 mgrid(std::min((lm->n_rows + kMergeThreads / 32 - 1) / (kMergeThreads / 32), dev.sm_count * 8));
     if (a.kmax == 0) e = launch_pdl(lmhead_merge_kernel<0>, mgrid, dim3(kMergeThreads), 0, s, a);
+    else if (a.kmax == 12) e = launch_pdl(lmhead_merge_kernel<12>, mgrid, dim3(kMergeThreads), 0, s, a);
     else if (a.kmax == 16) e = launch_pdl(lmhead_merge_kernel<16>, mgrid, dim3(kMergeThreads), 0, s, a);
     else e = launch_pdl(lmhead_merge_kernel<32>, mgrid, dim3(kMergeThreads), 0, s, a);
     return e == cudaSuccess ? RPS_OK : RPS_ERR_CUDA;

@@ -78,6 +78,29 @@ def check(h_bits, w_bits, k, rows=None):
     return err.max()
 
 
+@pytest.mark.parametrize("n,d,V,k", [
+    (129, 64, 516, 10),      # a pair with one row in its second half, one K slice, a four-token granule
+    (256, 320, 40000, 10),   # whole row tiles; ranges that end in half a vocabulary tile
+    (260, 192, 40004, 32),   # an odd number of row tiles: the last pair's second half is empty
+    (700, 128, 126464, 0),   # three pairs, several tiles each
+])
+def test_lmhead_pairs(n, d, V, k):
+    """Two row tiles or more: a pair of CTAs per tile. Row-major and packed unembedding alike."""
+    h, w = synth.lmhead_inputs(19, n, V, d)
+    rows = np.unique(np.r_[0, 127, 128, n - 1, np.linspace(0, n - 1, 24).astype(int)])
+    check(h, w, k, rows=rows)
+    out, lg, ws = run_lmhead(h, w, k)
+    wd = dev_bf16(w)
+    packed = rps.RowStatsBuf.alloc(n, k, "cuda")
+    lp = torch.empty_like(lg)
+    rps.rps_lmhead_row_stats(dev_bf16(h), wd, Prm(k) if k else None, packed, ws, lp,
+                             packed=rps.rps_lmhead_pack_unembed(wd))
+    assert rps.rps_poll_device_status() == (rps.RPS_OK, 0)
+    assert torch.equal(lg, lp)
+    for f in ("zmax", "lse", "H", "pmax", "argmax") + (("mu", "htrunc", "topk_idx", "topk_logit") if k else ()):
+        assert torch.equal(getattr(out, f), getattr(packed, f)), f
+
+
 @pytest.mark.parametrize("n,V,k,zero", [
     (1300, 9000, 20, 0),   # 13 splits for 20 ranks: the bound is taken two entries deep
     (5, 300, 32, 0),       # two splits: the bound at the lists' last entries
