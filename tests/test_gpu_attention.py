@@ -63,6 +63,11 @@ def check(q, k, v, C, NB, G, scale):
     (2, 4, 512, 9, 256),   # the lookahead shape: context 512, anchor + 8 branches of 256
     (3, 8, 0, 9, 96),      # one key tile per item, several items per CTA: every tile ends an item
     (4, 16, 64, 5, 64),    # two key tiles per item, two or three items per CTA
+    (2, 8, 328, 9, 32),    # four branches a tile, the last tile with one; four key tiles
+    (1, 24, 0, 17, 8),     # no context: sixteen branches a tile, one in the last; one key tile
+    (5, 16, 136, 7, 24),   # five branches of 24 a tile (120 rows), two in the last
+    (2, 40, 0, 2, 200),    # two key tiles per item, the second short, several items per CTA
+    (1, 40, 256, 3, 72),   # one branch per tile, just above half of it
 ])
 def test_packed_attention_parity(n_b, n_h, C, NB, G):
     q, k, v = inputs(31, n_b, n_h, C, NB, G)
