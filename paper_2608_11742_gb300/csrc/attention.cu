@@ -44,7 +44,6 @@
 // two run at once. 8 x 32 heads, context 512, 9 branches of 256: 266 -> 256 us;
 // 32 heads, context 328, 9 branches of 32: 20.4 -> 14.7 us (against two halves
 // of each row in turn with separate S and P V issuers, and a tile per branch).
-// PLACEHOLDER
 // Every wait is bounded; a role whose wait runs out flags RPS_DEVERR_TIMEOUT
 // and raises the CTA's abort flag, copies and MMAs in flight are drained and
 // TMEM is freed before the CTA exits.

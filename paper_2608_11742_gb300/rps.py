@@ -13,7 +13,8 @@ one decoding step together on preallocated buffers.
 from __future__ import annotations
 
 import ctypes as C
-from dataclasses import dataclass, fields
+from dataclasses import dataclass
+from operator import attrgetter
 from pathlib import Path
 from typing import Optional
 
@@ -101,9 +102,9 @@ _lib.rps_score_and_commit.argtypes = [C.POINTER(RpsLogits), C.c_int32, C.POINTER
                                       C.POINTER(RpsRowStats), C.c_int32, C.c_int32, C.POINTER(RpsPivots),
                                       C.POINTER(RpsParams), C.POINTER(RpsBranchScores), C.POINTER(RpsCommitOut), _p]
 _lib.rps_run_step.restype = C.c_int
-_lib.rps_run_step.argtypes = [C.POINTER(RpsLogits), C.c_int32, C.c_int32, _p, _p, C.POINTER(RpsParams),
-                              C.POINTER(RpsRowStats), C.POINTER(RpsPivots), C.POINTER(RpsRowStats),
-                              C.POINTER(RpsBranchScores), C.POINTER(RpsCommitOut), _p, C.c_size_t, _p, C.c_size_t, _p]
+# (structs by address: an integer converts in half the time of a byref)
+_lib.rps_run_step.argtypes = [_p, C.c_int32, C.c_int32, _p, _p, _p, _p, _p, _p, _p, _p, _p, C.c_size_t, _p, C.c_size_t,
+                              _p]
 _lib.rps_decode_advance.restype = C.c_int
 _lib.rps_decode_advance.argtypes = [C.POINTER(RpsPivots), C.POINTER(RpsCommitOut), C.c_int32, C.c_int32, C.c_int32,
                                     _p, _p, _p, _p, _p, _p, _p]
@@ -168,23 +169,57 @@ def params(p) -> RpsParams:
                      getattr(p, "pivot_rule", 0), getattr(p, "commit_rule", 0), getattr(p, "commit_k", 0))
 
 
+_data_ptr = torch.Tensor.data_ptr
+
+
+class _CStruct:
+    """A buffer set whose C struct is kept between calls: built field by field on each
+    one, a step's five took a third of its time on the host (48 us a call, 33 with
+    kept ones; the device takes 31 over the smallest step). Only the tensors'
+    addresses are read each time: the kept struct is used while they are all the
+    same, and built anew when a tensor was replaced, set or resized."""
+
+    __slots__ = ("_kept",)  # (addresses, struct)
+
+    def _c(self):
+        tensors = self._tensors(self)
+        try:
+            ptrs = list(map(_data_ptr, tensors)) if tensors[-1] is not None else None
+        except TypeError:
+            ptrs = None
+        if ptrs is None:  # (a form without some of the fields)
+            ptrs = [None if t is None else t.data_ptr() for t in tensors]
+        kept = getattr(self, "_kept", None)
+        if kept is None or kept[0] != ptrs:
+            kept = self._kept = (ptrs, self._struct(*ptrs))
+        return kept[1]
+
+    def __getstate__(self):  # a copy or a pickle holds the tensors alone
+        return self.__dict__
+
+    def c(self):
+        """The C struct of the buffers' present addresses."""
+        return self._struct(*[None if t is None else t.data_ptr() for t in self._tensors(self)])
+
+
 def logits_desc(t: torch.Tensor) -> RpsLogits:
     """Descriptor of a ``[n_req][n_branch][n_pos][vocab]`` bf16 / fp32 CUDA tensor."""
-    if t.dim() != 4 or t.stride(3) != 1:
+    shape, stride, dtype = t.shape, t.stride(), t.dtype
+    if len(shape) != 4 or stride[3] != 1:
         raise ValueError("logits must be 4-D with a contiguous vocab dimension")
-    if t.dtype == torch.bfloat16:
+    if dtype == torch.bfloat16:
         dt = RPS_BF16
-    elif t.dtype == torch.float32:
+    elif dtype == torch.float32:
         dt = RPS_F32
     else:
-        raise TypeError(f"logits must be bf16 or fp32, got {t.dtype}")
-    n_req, nb, L, V = t.shape
-    return RpsLogits(t.data_ptr(), dt, n_req, nb, L, V, t.stride(0), t.stride(1), t.stride(2))
+        raise TypeError(f"logits must be bf16 or fp32, got {dtype}")
+    n_req, nb, L, V = shape
+    return RpsLogits(t.data_ptr(), dt, n_req, nb, L, V, stride[0], stride[1], stride[2])
 
 
 # --------------------------------------------------------------------------- buffers
 @dataclass
-class RowStatsBuf:
+class RowStatsBuf(_CStruct):
     zmax: torch.Tensor
     lse: torch.Tensor
     H: torch.Tensor
@@ -203,12 +238,10 @@ class RowStatsBuf:
             return RowStatsBuf(f(n), f(n), f(n), f(n), i(n), f(n), f(n), i(n, k), f(n, k))
         return RowStatsBuf(f(n), f(n), f(n), f(n), i(n))
 
-    def c(self) -> RpsRowStats:
-        return RpsRowStats(*(_ptr(getattr(self, f.name)) for f in fields(self)))
 
 
 @dataclass
-class PivotsBuf:
+class PivotsBuf(_CStruct):
     n_commit: torch.Tensor
     commit_pos: torch.Tensor
     commit_tok: torch.Tensor
@@ -235,12 +268,10 @@ class PivotsBuf:
                          torch.zeros(n_req, NB, dtype=torch.uint8, device=device), i(n_req, NB), i(n_req, NB),
                          i(n_req), i(n_req, NB * L, 3))
 
-    def c(self) -> RpsPivots:
-        return RpsPivots(*(_ptr(getattr(self, n)) for n in _PIVOT_FIELDS))
 
 
 @dataclass
-class ScoresBuf:
+class ScoresBuf(_CStruct):
     mean_H: torch.Tensor
     n_tau: torch.Tensor
     log_a: torch.Tensor
@@ -251,12 +282,10 @@ class ScoresBuf:
         f = lambda: torch.full((n_req, P, K + 1), float("nan"), dtype=torch.float32, device=device)
         return ScoresBuf(f(), torch.full((n_req, P, K + 1), -1, dtype=torch.int32, device=device), f(), f())
 
-    def c(self) -> RpsBranchScores:
-        return RpsBranchScores(*(_ptr(getattr(self, f.name)) for f in fields(self)))
 
 
 @dataclass
-class CommitBuf:
+class CommitBuf(_CStruct):
     best_slot: torch.Tensor
     gain: torch.Tensor
     winner: torch.Tensor
@@ -272,8 +301,17 @@ class CommitBuf:
         f = lambda *s: torch.full(s, float("nan"), dtype=torch.float32, device=device)
         return CommitBuf(i(n_req, P), f(n_req, P), i(n_req), i(n_req), i(n_req), f(n_req), i(n_req, L), i(n_req))
 
-    def c(self) -> RpsCommitOut:
-        return RpsCommitOut(*(_ptr(getattr(self, f.name)) for f in fields(self)))
+
+
+for _cls, _st in ((RowStatsBuf, RpsRowStats), (PivotsBuf, RpsPivots), (ScoresBuf, RpsBranchScores),
+                  (CommitBuf, RpsCommitOut)):
+    _cls._struct = _st
+    _cls._tensors = attrgetter(*(n for n, _ in _st._fields_))
+
+
+def _cs(buf):
+    """The C struct of a buffer set (any object with ``c()`` will do)."""
+    return buf._c() if isinstance(buf, _CStruct) else buf.c()
 
 
 # --------------------------------------------------------------------------- ABI calls
@@ -312,7 +350,7 @@ def rps_score_step(logits: torch.Tensor, rows: Optional[torch.Tensor], seg_cnt: 
     desc = logits_desc(logits)
     rl = RpsRowList(_ptr(rows), _ptr(seg_cnt), n_seg, cap, _ptr(mask_pos), mask_branch)
     p = params(prm)
-    st = out.c()
+    st = _cs(out)
     _check(_lib.rps_score_step(C.byref(desc), C.byref(rl), C.byref(p), C.byref(st), ws.data_ptr(),
                                ws.numel() * ws.element_size(), _stream(stream)), "rps_score_step")
 
@@ -325,7 +363,7 @@ def rps_score_step_noalloc(logits: torch.Tensor, rows: Optional[torch.Tensor], s
     desc = logits_desc(logits)
     rl = RpsRowList(_ptr(rows), _ptr(seg_cnt), n_seg, cap, _ptr(mask_pos), mask_branch)
     p = params(prm)
-    st = out.c()
+    st = _cs(out)
     _check(_lib.rps_score_step_noalloc(C.byref(desc), C.byref(rl), C.byref(p), C.byref(st), _stream(stream)),
            "rps_score_step_noalloc")
 
@@ -346,20 +384,20 @@ def rps_gather_rows(src: torch.Tensor, rows: Optional[torch.Tensor], seg_cnt: Op
 
 def rps_select_pivots(base: RowStatsBuf, n_req: int, L: int, mask_pos: torch.Tensor, mask_cnt: torch.Tensor, prm,
                       out: PivotsBuf, stream=None) -> None:
-    b, p, o = base.c(), params(prm), out.c()
+    b, p, o = _cs(base), params(prm), _cs(out)
     _check(_lib.rps_select_pivots(C.byref(b), n_req, L, mask_pos.data_ptr(), mask_cnt.data_ptr(), C.byref(p),
                                   C.byref(o), _stream(stream)), "rps_select_pivots")
 
 
 def rps_score_branches(anchor_logits: torch.Tensor, anchor_branch: int, anchor: RowStatsBuf, branch: RowStatsBuf,
                        n_req: int, L: int, piv: PivotsBuf, prm, out: ScoresBuf, stream=None) -> None:
-    d, a, b, pv, p, o = logits_desc(anchor_logits), anchor.c(), branch.c(), piv.c(), params(prm), out.c()
+    d, a, b, pv, p, o = logits_desc(anchor_logits), _cs(anchor), _cs(branch), _cs(piv), params(prm), _cs(out)
     _check(_lib.rps_score_branches(C.byref(d), anchor_branch, C.byref(a), C.byref(b), n_req, L, C.byref(pv),
                                    C.byref(p), C.byref(o), _stream(stream)), "rps_score_branches")
 
 
 def rps_commit(scores: ScoresBuf, n_req: int, L: int, piv: PivotsBuf, prm, out: CommitBuf, stream=None) -> None:
-    s, pv, p, o = scores.c(), piv.c(), params(prm), out.c()
+    s, pv, p, o = _cs(scores), _cs(piv), params(prm), _cs(out)
     _check(_lib.rps_commit(C.byref(s), n_req, L, C.byref(pv), C.byref(p), C.byref(o), _stream(stream)),
            "rps_commit")
 
@@ -367,8 +405,8 @@ def rps_commit(scores: ScoresBuf, n_req: int, L: int, piv: PivotsBuf, prm, out: 
 def rps_score_and_commit(anchor_logits: torch.Tensor, anchor_branch: int, anchor: RowStatsBuf, branch: RowStatsBuf,
                          n_req: int, L: int, piv: PivotsBuf, prm, scores: ScoresBuf, out: CommitBuf,
                          stream=None) -> None:
-    d, a, b, pv, p = logits_desc(anchor_logits), anchor.c(), branch.c(), piv.c(), params(prm)
-    s, o = scores.c(), out.c()
+    d, a, b, pv, p = logits_desc(anchor_logits), _cs(anchor), _cs(branch), _cs(piv), params(prm)
+    s, o = _cs(scores), _cs(out)
     _check(_lib.rps_score_and_commit(C.byref(d), anchor_branch, C.byref(a), C.byref(b), n_req, L, C.byref(pv),
                                      C.byref(p), C.byref(s), C.byref(o), _stream(stream)), "rps_score_and_commit")
 
@@ -377,16 +415,17 @@ def rps_run_step(logits: torch.Tensor, n_req: int, L: int, mask_pos: torch.Tenso
                  base: RowStatsBuf, piv: PivotsBuf, branch: RowStatsBuf, scores: ScoresBuf, out: CommitBuf,
                  ws_base: torch.Tensor, ws_branch: torch.Tensor, stream=None) -> None:
     d, p = logits_desc(logits), params(prm)
-    b, pv, br, sc, o = base.c(), piv.c(), branch.c(), scores.c(), out.c()
-    _check(_lib.rps_run_step(C.byref(d), n_req, L, mask_pos.data_ptr(), mask_cnt.data_ptr(), C.byref(p), C.byref(b),
-                             C.byref(pv), C.byref(br), C.byref(sc), C.byref(o), ws_base.data_ptr(),
-                             ws_base.numel() * ws_base.element_size(), ws_branch.data_ptr(),
-                             ws_branch.numel() * ws_branch.element_size(), _stream(stream)), "rps_run_step")
+    b, pv, br, sc, o = _cs(base), _cs(piv), _cs(branch), _cs(scores), _cs(out)
+    at = C.addressof
+    _check(_lib.rps_run_step(at(d), n_req, L, mask_pos.data_ptr(), mask_cnt.data_ptr(), at(p), at(b), at(pv), at(br),
+                             at(sc), at(o), ws_base.data_ptr(), ws_base.numel() * ws_base.element_size(),
+                             ws_branch.data_ptr(), ws_branch.numel() * ws_branch.element_size(), _stream(stream)),
+           "rps_run_step")
 
 
 def rps_decode_advance(piv: PivotsBuf, commit: CommitBuf, n_req: int, B: int, L_total: int, tokens, block, mask_pos,
                        mask_cnt, done, steps=None, stream=None) -> None:
-    pv, cm = piv.c(), commit.c()
+    pv, cm = _cs(piv), _cs(commit)
     _check(_lib.rps_decode_advance(C.byref(pv), C.byref(cm), n_req, B, L_total, tokens.data_ptr(), block.data_ptr(),
                                    mask_pos.data_ptr(), mask_cnt.data_ptr(), done.data_ptr(),
                                    None if steps is None else steps.data_ptr(), _stream(stream)),
@@ -437,7 +476,7 @@ def rps_lmhead_row_stats(hidden: torch.Tensor, unembed: torch.Tensor, prm, out: 
     lm = RpsLmhead(hidden.data_ptr(), src, hidden.shape[0], hidden.shape[1], unembed.shape[0],
                    hidden.stride(0), unembed.stride(0), 0 if packed is None else 1)
     p = params(prm) if prm is not None else None
-    st = out.c()
+    st = _cs(out)
     _check(_lib.rps_lmhead_row_stats(C.byref(lm), None if p is None else C.byref(p), C.byref(st), _ptr(logits_out),
                                      ws.data_ptr(), ws.numel() * ws.element_size(), _stream(stream)),
            "rps_lmhead_row_stats")
@@ -447,11 +486,13 @@ def rps_packed_attention_fwd(q: torch.Tensor, k: torch.Tensor, vt: torch.Tensor,
                              n_branch: int, branch_len: int, scale: float, stream=None) -> None:
     """Branch-isolating attention of a packed lookahead sequence: q, k, out
     ``[batch][heads][tokens][128]`` and vt ``[batch][heads][128][tokens]``, bf16 CUDA tensors."""
+    bf16 = torch.bfloat16
     for t in (q, k, vt, out):
-        if t.dtype != torch.bfloat16 or not t.is_contiguous() or t.dim() != 4:
+        if t.dtype != bf16 or not t.is_contiguous() or t.dim() != 4:
             raise ValueError("q, k, vt and out must be contiguous 4-D bf16 tensors")
-    n_b, n_h, n_tok, d = q.shape
-    if k.shape != q.shape or out.shape != q.shape or vt.shape != (n_b, n_h, d, n_tok):
+    shape = q.shape
+    n_b, n_h, n_tok, d = shape
+    if k.shape != shape or out.shape != shape or vt.shape != (n_b, n_h, d, n_tok):
         raise ValueError("shapes: q, k, out [b][h][tokens][d] and vt [b][h][d][tokens]")
     if n_tok != n_context + n_branch * branch_len:
         raise ValueError("tokens must be n_context + n_branch * branch_len")
