@@ -10,8 +10,9 @@
 namespace rps {
 namespace {
 
-// a.early: the mask predates the previous launch (the base rows' statistics),
-// so it is staged before waiting for that launch. The next launch (the
+// a.early: the previous launch on the stream is the base rows' top-k search, so
+// what that one does not write (the mask, the rows' P^max and entropy) is read,
+// and M split, before waiting for it. The next launch (the
 // lookahead rows' statistics) is released only at the end: its blocks would
 // otherwise sit, waiting, on this block's SM while it works.
 __global__ void __launch_bounds__(kSelectThreads) select_kernel(const SelectArgs a) {

@@ -126,7 +126,7 @@ __device__ void block_top_keys(const uint64_t *keys, int n, int P, uint64_t *t_a
 }
 
 // Dynamic shared memory of select_kernel: per masked position, then a constant.
-constexpr int kSelectBytesPerPos = sizeof(uint64_t) + sizeof(uint64_t) + 4 * sizeof(float) + 4 * sizeof(int32_t) + 1;
+constexpr int kSelectBytesPerPos = sizeof(uint64_t) + sizeof(uint64_t) + 2 * sizeof(float) + 4 * sizeof(int32_t) + 1;
 constexpr int kSelectBytesExtra = 2 * 32 * sizeof(uint64_t) + 16;
 __host__ __device__ constexpr int half_keys(int L) { return L / 2 + 32; }
 
@@ -151,9 +151,12 @@ __host__ __device__ constexpr size_t select_smem_bytes(int L) {
 // Steps 1-6 of one request (standard commit, M', pivots, candidates, lookahead
 // rows) by one block of at most kSelectThreads threads, in `smem` of
 // select_smem_bytes(L). The statistics are read through L2 (__ldcg). With
-// `wait_inside` the block calls pdl_wait itself after staging the mask and
-// writing the defaults: the base statistics are the only input the previous
-// launch writes.
+// `wait_inside` the block calls pdl_wait itself, after the split of M into S and
+// M': the previous launch is the base rows' top-k search, which writes their
+// argmax, mu, truncated entropy and lists; their P^max, H and zmax come from the
+// launch before it, which was complete when that one let this one begin. (The
+// split takes 1.3 us, about as long as the search's last rows.) Each thread
+// waits before it returns: the next launch counts on this one ending last.
 __device__ void select_request(const SelectArgs &a, int q, unsigned char *smem, bool wait_inside) {
     const int tid = threadIdx.x;
     const int L = a.L, P = a.P, K = a.K, NB = P * K;
@@ -173,12 +176,10 @@ __device__ void select_request(const SelectArgs &a, int q, unsigned char *smem, 
     uint64_t *t_a = keys + L;                                 // tournament buffers
     uint64_t *t_b = t_a + half_keys(L);
     float *pm = reinterpret_cast<float *>(t_b + half_keys(L));  // P^max of mask entry k
-    float *mu = pm + L;                                         // retained mass
-    float *ht = mu + L;                                         // truncated entropy
-    float *hh = ht + L;                                         // entropy
+    float *hh = pm + L;                                         // entropy
     int32_t *pos = reinterpret_cast<int32_t *>(hh + L);         // position
-    int32_t *am = pos + L;                                      // argmax token
-    int32_t *rk = am + L;                                       // M' entry i -> mask entry
+    int32_t *place = pos + L;                                   // mask entry -> M' entry, or ~ its place in S
+    int32_t *rk = place + L;                                    // M' entry i -> mask entry
     int32_t *rp = rk + L;                                       // M' entry i -> position
     uint8_t *in_S = reinterpret_cast<uint8_t *>(rp + L);
 
@@ -202,20 +203,9 @@ __device__ void select_request(const SelectArgs &a, int q, unsigned char *smem, 
         o.branch_off[q * NB + b] = 0;
         o.branch_cnt[q * NB + b] = 0;
     }
-    if (wait_inside) pdl_wait();
     for (int k = tid; k < L; k += blockDim.x) {
         pm[k] = __ldcg(a.pmax + base + k);
-        mu[k] = __ldcg(a.mu + base + k);
-        ht[k] = __ldcg(a.htrunc + base + k);
         hh[k] = __ldcg(a.H + base + k);
-        am[k] = __ldcg(a.argmax + base + k);
-        // the pivots' candidate step reads a row's zmax and top-k list: bring
-        // them to L1 now, while the statistics load, instead of a round trip later
-        if (k < cnt) {
-            prefetch_l1(a.zmax + base + k);
-            prefetch_l1(a.topk_logit + (base + k) * a.k_max);
-            prefetch_l1(a.topk_idx + (base + k) * a.k_max);
-        }
     }
     __syncthreads();
 
@@ -268,17 +258,12 @@ __device__ void select_request(const SelectArgs &a, int q, unsigned char *smem, 
         if (k < cnt) {
             if (f) {
                 o.commit_pos[base + n_commit + excl] = pos[k];
-                o.commit_tok[base + n_commit + excl] = am[k];
+                place[k] = ~(n_commit + excl);
             } else {
                 const int r = k - (n_commit + excl);
+                place[k] = r;
                 rk[r] = k;
                 rp[r] = pos[k];
-                if (a.pivot_rule == RPS_PIVOT_TRUNCATED_ENTROPY)
-                    keys[r] = mu[k] >= a.tau_pivot && ht[k] == ht[k] ? pivot_key(ht[k], pos[k]) : 0ull;
-                else {
-                    const float v = a.pivot_rule == RPS_PIVOT_MAX_CONFIDENCE ? pm[k] : hh[k];
-                    keys[r] = v == v ? pivot_key(v, pos[k]) : 0ull;
-                }
                 o.rem_k[base + r] = k;
                 o.rem_pos[base + r] = pos[k];
             }
@@ -290,6 +275,28 @@ __device__ void select_request(const SelectArgs &a, int q, unsigned char *smem, 
         o.n_commit[q] = n_commit;
         o.rem_cnt[q] = n_rem;
         o.n_branch_rows[q] = 0;
+    }
+
+    // What the top-k search wrote: the committed tokens and the pivot keys (each
+    // thread reads back the places it wrote itself).
+    if (wait_inside) pdl_wait();
+    for (int k = tid; k < cnt; k += blockDim.x) {
+        const float m = __ldcg(a.mu + base + k), h = __ldcg(a.htrunc + base + k);
+        const int32_t am = __ldcg(a.argmax + base + k);
+        // the pivots' candidate step reads a row's zmax and top-k list: bring
+        // them to L1 now, while these load, instead of a round trip later
+        prefetch_l1(a.zmax + base + k);
+        prefetch_l1(a.topk_logit + (base + k) * a.k_max);
+        prefetch_l1(a.topk_idx + (base + k) * a.k_max);
+        const int r = place[k];
+        if (r < 0) {
+            o.commit_tok[base + ~r] = am;
+        } else if (a.pivot_rule == RPS_PIVOT_TRUNCATED_ENTROPY) {
+            keys[r] = m >= a.tau_pivot && h == h ? pivot_key(h, pos[k]) : 0ull;
+        } else {
+            const float v = a.pivot_rule == RPS_PIVOT_MAX_CONFIDENCE ? pm[k] : hh[k];
+            keys[r] = v == v ? pivot_key(v, pos[k]) : 0ull;
+        }
     }
     if (n_rem == 0) {
         if (tid == 0) o.state[q] = RPS_STATE_DONE;

@@ -1146,12 +1146,14 @@ __global__ void __launch_bounds__(kTopkWarps * 32, kTopkMinBlocks) topk_rows_ker
     __shared__ uint4 stage_all[kTopkWarps][kBatch * 32];
     __shared__ float2 cand_all[kTopkWarps][kCandBatch];
     __shared__ int32_t cells_all[kTopkWarps][kCellCap];
+    __shared__ int32_t n_cells_all[kTopkWarps];
 
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
     uint4 *stage = stage_all[wib];
     float2 *cand = cand_all[wib];
     int32_t *cells = cells_all[wib];
+    int32_t *n_cells = &n_cells_all[wib];
     const int64_t n_slots = static_cast<int64_t>(a.n_seg) * a.cap;
     const int64_t nv = a.units_per_row;
     const int V = static_cast<int>(a.vocab);
@@ -1242,6 +1244,24 @@ __global__ void __launch_bounds__(kTopkWarps * 32, kTopkMinBlocks) topk_rows_ker
             for (int q = 0; q < kSketchVecs; ++q)
                 if (vm[q] >= theta) hv |= 1u << q;
             if (!__any_sync(kFull, hv != 0)) continue;
+            if (one_batch) {
+                // The usual case, all cells in the buffer: each lane takes places for
+                // its cells from a counter (their order does not matter), in one
+                // pass over its hit vectors.
+                if (lane == 0) *n_cells = 0;
+                __syncwarp();
+                for (uint32_t b = hv; b; b &= b - 1) {
+                    const int q = __ffs(b) - 1;
+                    uint32_t m = vector_hits<DT>(sk + q * 32 + lane, theta);
+                    int at = atomicAdd(n_cells, __popc(m));
+                    for (; m && at < kCellCap; m &= m - 1) cells[at++] = (q * 32 + lane) * kPerVec + __ffs(m) - 1;
+                }
+                __syncwarp();
+                pending = *n_cells;
+                if (pending <= kCellCap) break;
+                pending = 0;  // too many: in rounds, below
+                __syncwarp();
+            }
             int c = 0;
             for (uint32_t b = hv; b; b &= b - 1) c += __popc(vector_hits<DT>(sk + v0 + (__ffs(b) - 1) * 32 + lane, theta));
             int incl = c;

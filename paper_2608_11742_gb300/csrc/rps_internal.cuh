@@ -104,7 +104,7 @@ struct SelectArgs {
     int32_t pivot_rule, commit_rule, commit_k;
     rps_pivots out;
     uint32_t *err;
-    int32_t early;  // the mask predates the previous launch (see select_kernel)
+    int32_t early;  // the previous launch is the base rows' top-k search (see select_kernel)
 };
 
 struct ScoreArgs {
