@@ -604,6 +604,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 // the few candidates, one copy of the insertion (the list only
                 // grows stricter, so each is checked again against it), their
                 // logits picked by index from shared memory
+                if (!live) cand = 0;  // (rows past the last: equal logits, all of them candidates)
                 if (KMAX > 0 && __any_sync(kFull, cand != 0)) {
 #pragma unroll
                     for (int i = 0; i < 32; ++i) pick[i * (kEpiWarps * 32)] = v[i];
