@@ -98,6 +98,7 @@ struct __align__(16) LmPartial {
 
 struct LmArgs {
     int32_t n_rows, d, n_gran, splits, kmax, k;  // n_gran: granules of the vocabulary
+    int32_t h_rows;  // rows of a hidden copy: a tile's, or all of fewer
     const uint8_t *w_packed;  // unembedding in the packed tile layout, or nullptr (tensor map)
     int64_t vocab;
     LmPartial *part;   // [n_rows][splits]
@@ -362,6 +363,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int col_end = static_cast<int>(static_cast<int64_t>(split + 1) * a.n_gran / a.splits) * Sh::granule;
     const int n_tiles = (col_end - col_begin + kTileN - 1) / kTileN;
     const int kblocks = a.d / kTileK;
+    // With fewer rows than a tile the hidden copies are that high: filling most of
+    // a tile from outside so small a tensor is slow (V 126,464, d 4,096, k 10: 4 rows
+    // 235 -> 164 us; V 32,000, d 1,024: 28.4 -> 22.5). A last tile of several is filled
+    // with zeros at no cost, and a pair's empty half is zeroed once.
+    const int row0 = rt * kTileM;
+    const bool has_rows = row0 < a.n_rows;
+    const int h_bytes = a.h_rows * kTileK * 2;  // of one slice
     // the ring starts on a 1024-byte boundary (the 128-byte swizzle's period)
     uint8_t *ring = dyn_smem + ((1024u - (saddr(dyn_smem) & 1023u)) & 1023u);
 
@@ -386,6 +394,13 @@ __global__ void __launch_bounds__(kThreads, 1)
         tmem_alloc<CG>(&c.tmem_base, kTmemCols);
         tmem_relinquish<CG>();
     }
+    if (CG == 2 && !has_rows) {
+        for (int i = threadIdx.x; i < kStages * Sh::slices * kABytes / 16; i += kThreads) {
+            constexpr int kPerStage = Sh::slices * kABytes / 16;
+            *reinterpret_cast<uint4 *>(ring + i / kPerStage * kStageBytes + i % kPerStage * 16) = make_uint4(0, 0, 0, 0);
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
     // the hidden rows may come from the previous kernel on the stream
     pdl_wait();
     pdl_launch_next();
@@ -402,6 +417,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (threadIdx.x == 0) flag_error(a.err, RPS_DEVERR_WORKSPACE);
     } else if (warp == 0) {
         if (lane == 0) {  // ---------------------------------------- TMA producer
+            const int pair_tiles = (rt | 1) * kTileM < a.n_rows ? 2 : 1;  // row tiles of the pair (CG 2)
             uint32_t it = 0;
             bool ok = true;
             for (int t = 0; t < n_tiles && ok; ++t) {
@@ -416,8 +432,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
                     uint8_t *sa = ring + s * kStageBytes;
                     if constexpr (CG == 1) {
-                        mbar_expect_tx(&c.full[s], kStageBytes);
-                        tma_load_2d(sa, &tm_h, kb * kTileK, rt * kTileM, &c.full[s]);
+                        mbar_expect_tx(&c.full[s], h_bytes + kBBytes);
+                        tma_load_2d(sa, &tm_h, kb * kTileK, row0, &c.full[s]);
                         if (a.w_packed)  // one contiguous 32 KB block, already in the swizzled image
                             bulk_load(sa + kABytes,
                                       a.w_packed + (static_cast<int64_t>(col0 / kTileN) * kblocks + kb) * kBBytes, kBBytes,
@@ -429,10 +445,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                         // expects the bytes of both
                         const uint32_t bar = leader_addr(&c.full[s]);
                         if (rank == 0)
-                            mbar_expect_tx(&c.full[s], Sh::slices * (2 * kABytes + n_cols * kTileK * 2));
+                            mbar_expect_tx(&c.full[s], Sh::slices * (h_bytes * pair_tiles + n_cols * kTileK * 2));
                         // one copy per operand for all slices of the stage (past the last
                         // slice of d it brings values that no MMA reads)
-                        tma_load_3d_pair(sa, &tm_h, 0, rt * kTileM, kb, bar);
+                        if (has_rows) tma_load_3d_pair(sa, &tm_h, 0, row0, kb, bar);
                         const int tok = col0 + rank * (n_cols / 2);  // this CTA's half of the tile's tokens
                         const CUtensorMap *map = n_cols == kTileN ? &tm_w : &tm_w_half;
                         uint8_t *sb = sa + Sh::slices * kABytes;
@@ -496,7 +512,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         __syncwarp();
     } else {  // ---------------------------------------------------- epilogue
         const int q = warp & 3;  // this warp's quarter of the TMEM lanes
-        const int row = rt * kTileM + q * 32 + lane;
+        const int row = row0 + q * 32 + lane;
         const bool live = row < a.n_rows;
         RowState<KMAX> st;
         st.B = -INFINITY;
@@ -1086,7 +1102,7 @@ rps_status rps_lmhead_row_stats(const rps_lmhead *lm, const rps_params *prm, con
     LmMaps maps;
     std::memset(&maps, 0, sizeof maps);
     if (pair) {
-        st = make_slice_map(&maps.h, lm->hidden, lm->n_rows, lm->d, lm->hidden_stride, kTileM);
+        st = make_slice_map(&maps.h, lm->hidden, lm->n_rows, lm->d, lm->hidden_stride, kTileM);  // (n_rows > kTileM)
         for (int half = 0; half < 2 && st == RPS_OK; ++half) {
             CUtensorMap *m = half ? &maps.w_half : &maps.w;
             const int rows = kTileN / 2 >> half;  // one CTA's tokens
@@ -1095,7 +1111,8 @@ rps_status rps_lmhead_row_stats(const rps_lmhead *lm, const rps_params *prm, con
         }
         if (st != RPS_OK) return st;
     } else {
-        if ((st = make_map(&maps.h, lm->hidden, lm->n_rows, lm->d, lm->hidden_stride, kTileM)) != RPS_OK) return st;
+        st = make_map(&maps.h, lm->hidden, lm->n_rows, lm->d, lm->hidden_stride, std::min<int32_t>(lm->n_rows, kTileM));
+        if (st != RPS_OK) return st;
         maps.w = maps.h;  // (single CTAs read the packed unembedding without a tensor map)
         if (!lm->unembed_packed &&
             (st = make_map(&maps.w, lm->unembed, lm->vocab, lm->d, lm->unembed_stride, kTileN)) != RPS_OK)
@@ -1105,6 +1122,7 @@ rps_status rps_lmhead_row_stats(const rps_lmhead *lm, const rps_params *prm, con
     LmArgs a;
     std::memset(&a, 0, sizeof a);
     a.n_rows = lm->n_rows;
+    a.h_rows = std::min<int32_t>(lm->n_rows, kTileM);
     a.d = lm->d;
     a.splits = splits;
     a.kmax = list_len(k);
