@@ -228,6 +228,8 @@ rps_status prepare_row_stats(const rps_logits *logits, const rps_row_list *rows,
     a.min_piece = std::max<int64_t>((a.units_per_row + (kMaxPartials - 2) - 1) / (kMaxPartials - 2),
                                     std::min<int64_t>(a.units_per_row, 32 * kBatch));
     a.max_ppr = static_cast<int32_t>((a.units_per_row + a.min_piece - 1) / a.min_piece);
+    // a row lies in at most max_ppr + 1 pieces, each of which may end in a partial chunk
+    a.few_chunks = a.units_per_row / (32 * kBatch) + a.max_ppr + 1 <= kFewChunks;
     a.err = dev.err;
     *grid_out = grid;
     return RPS_OK;

@@ -207,6 +207,7 @@ struct Elem<RPS_BF16> {
     typedef uint16_t Sketch;
     static constexpr uint32_t kNegInf2 = 0xff80ff80u;  // a 32-bit word of -inf sketch entries
     __device__ static __forceinline__ Sketch to_sketch(float v) { return static_cast<uint16_t>(__float_as_uint(v) >> 16); }
+    __device__ static __forceinline__ float from_sketch(Sketch v) { return __uint_as_float(static_cast<uint32_t>(v) << 16); }
     // running maximum of whole units, kept as a packed bf16 pair
     typedef uint32_t Acc;
     __device__ static __forceinline__ Acc acc_init() { return 0xff80ff80u; }  // (-inf, -inf)
@@ -242,6 +243,7 @@ struct Elem<RPS_F32> {
     typedef float Sketch;
     static constexpr uint32_t kNegInf2 = 0xff800000u;
     __device__ static __forceinline__ Sketch to_sketch(float v) { return v; }
+    __device__ static __forceinline__ float from_sketch(Sketch v) { return v; }
     typedef float Acc;
     __device__ static __forceinline__ Acc acc_init() { return -INFINITY; }
     __device__ static __forceinline__ Acc acc_add(Acc m, const uint4 &w) { return fmaxf(m, unit_max(w)); }
@@ -1139,7 +1141,30 @@ __device__ __forceinline__ uint32_t vector_hits(const uint4 *p, float theta) {
     return m;
 }
 
+// vector_hits of sketch vector v, without the entries past the row's chunks when
+// theta is -inf (they read as -inf).
 template <int DT>
+__device__ __forceinline__ uint32_t cell_hits(const uint4 *sk, int v, float theta, const SketchRow &cut, int full_units) {
+    constexpr int kPerVec = 16 / static_cast<int>(sizeof(typename Elem<DT>::Sketch));
+    uint32_t m = vector_hits<DT>(sk + v, theta);
+    if (theta == -INFINITY) {
+        for (uint32_t b = m; b; b &= b - 1) {
+            int first, count;
+            sketch_cell(cut, full_units, v * kPerVec + __ffs(b) - 1, first, count);
+            if (count == 0) m &= ~(b & (0u - b));
+        }
+    }
+    return m;
+}
+
+// FEW: rows of at most kFewChunks ring chunks. One sketch entry per lane and chunk fits
+// the registers, so the bound is taken over cells (each lane's largest two)
+// instead of vectors of them, and the hits need no second look. A short row has
+// too few vectors: V 3,447 has 16, so that at k = 32 every cell was reloaded (64
+// rows: 434 us, here 13; k = 16 at V 2,100 26.6 -> 10.8, k = 10 the same).
+static_assert(kFewChunks <= 32, "one hit bit per chunk");
+
+template <int DT, bool FEW>
 __global__ void __launch_bounds__(kTopkWarps * 32, kTopkMinBlocks) topk_rows_kernel(const RowStatsArgs a) {
     using E = Elem<DT>;
     constexpr int kPerVec = 16 / static_cast<int>(sizeof(typename E::Sketch));  // sketch entries per 16 bytes
@@ -1191,9 +1216,17 @@ __global__ void __launch_bounds__(kTopkWarps * 32, kTopkMinBlocks) topk_rows_ker
         const float4 nrm = __ldcg(a.norm + slot);
         const int piece = __ldcg(a.sketch_piece);
         const uint32_t health = __ldcg(a.health);
-        // Pass 1: the largest entry of each of this lane's vectors v0 + 32 q + lane.
-        float vm[kSketchVecs];
-        vector_maxima<DT>(vm, sk, 0, n_vec, lane);
+        // Pass 1: the largest entry of each of this lane's vectors v0 + 32 q + lane
+        // (short rows: its entry of each chunk).
+        float vm[kSketchVecs], em[FEW ? kFewChunks : 1];
+        if constexpr (FEW) {
+            const typename E::Sketch *entries = reinterpret_cast<const typename E::Sketch *>(sk);
+#pragma unroll
+            for (int c = 0; c < kFewChunks; ++c)
+                em[c] = c * 32 < a.sketch_stride ? E::from_sketch(__ldg(entries + c * 32 + lane)) : -INFINITY;
+        } else {
+            vector_maxima<DT>(vm, sk, 0, n_vec, lane);
+        }
         if (health != 0) {  // the statistics launch gave up, or found the workspace unhealthy
             if (lane == 0) flag_error(a.err, RPS_DEVERR_WORKSPACE);
             break;
@@ -1218,7 +1251,14 @@ __global__ void __launch_bounds__(kTopkWarps * 32, kTopkMinBlocks) topk_rows_ker
         // the k-th largest of the lanes' largest entries
         // (for long lists, of each lane's two largest vectors' maxima)
         float lane_max = -INFINITY, lane_2nd = -INFINITY;
-        for (int v0 = 0;;) {
+        if constexpr (FEW) {
+#pragma unroll
+            for (int c = 0; c < kFewChunks; ++c) {
+                lane_2nd = fmaxf(lane_2nd, fminf(lane_max, em[c]));
+                lane_max = fmaxf(lane_max, em[c]);
+            }
+        }
+        for (int v0 = 0; !FEW;) {
 #pragma unroll
             for (int q = 0; q < kSketchVecs; ++q) {
                 lane_2nd = fmaxf(lane_2nd, fminf(lane_max, vm[q]));
@@ -1237,8 +1277,30 @@ __global__ void __launch_bounds__(kTopkWarps * 32, kTopkMinBlocks) topk_rows_ker
         int ti = INT_MAX;
         bool empty = true;
         int pending = 0;
-        for (int v0 = 0; v0 < n_vec; v0 += 32 * kSketchVecs) {
-            if (!one_batch) vector_maxima<DT>(vm, sk, v0, n_vec, lane);
+        bool listed = false;
+        if constexpr (FEW) {
+            uint32_t he = 0;  // bit c: this lane's entry of chunk c reaches theta
+#pragma unroll
+            for (int c = 0; c < kFewChunks; ++c)
+                if (em[c] >= theta) he |= 1u << c;
+            if (theta == -INFINITY) {  // (not the entries past the row's chunks)
+                for (uint32_t b = he; b; b &= b - 1) {
+                    int first, count;
+                    sketch_cell(cut, full_units, (__ffs(b) - 1) * 32 + lane, first, count);
+                    if (count == 0) he &= ~(b & (0u - b));
+                }
+            }
+            if (lane == 0) *n_cells = 0;
+            __syncwarp();
+            int at = he ? atomicAdd(n_cells, __popc(he)) : 0;
+            for (; he && at < kCellCap; he &= he - 1) cells[at++] = (__ffs(he) - 1) * 32 + lane;
+            __syncwarp();
+            listed = *n_cells <= kCellCap;
+            if (listed) pending = *n_cells;  // else in rounds, as vectors
+            __syncwarp();
+        }
+        for (int v0 = 0; v0 < n_vec && !listed; v0 += 32 * kSketchVecs) {
+            if (!one_batch || FEW) vector_maxima<DT>(vm, sk, v0, n_vec, lane);
             uint32_t hv = 0;  // bit q: vector q holds an entry at or above theta
 #pragma unroll
             for (int q = 0; q < kSketchVecs; ++q)
@@ -1252,7 +1314,7 @@ __global__ void __launch_bounds__(kTopkWarps * 32, kTopkMinBlocks) topk_rows_ker
                 __syncwarp();
                 for (uint32_t b = hv; b; b &= b - 1) {
                     const int q = __ffs(b) - 1;
-                    uint32_t m = vector_hits<DT>(sk + q * 32 + lane, theta);
+                    uint32_t m = cell_hits<DT>(sk, q * 32 + lane, theta, cut, full_units);
                     int at = atomicAdd(n_cells, __popc(m));
                     for (; m && at < kCellCap; m &= m - 1) cells[at++] = (q * 32 + lane) * kPerVec + __ffs(m) - 1;
                 }
@@ -1263,7 +1325,7 @@ __global__ void __launch_bounds__(kTopkWarps * 32, kTopkMinBlocks) topk_rows_ker
                 __syncwarp();
             }
             int c = 0;
-            for (uint32_t b = hv; b; b &= b - 1) c += __popc(vector_hits<DT>(sk + v0 + (__ffs(b) - 1) * 32 + lane, theta));
+            for (uint32_t b = hv; b; b &= b - 1) c += __popc(cell_hits<DT>(sk, v0 + (__ffs(b) - 1) * 32 + lane, theta, cut, full_units));
             int incl = c;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
@@ -1275,7 +1337,7 @@ __global__ void __launch_bounds__(kTopkWarps * 32, kTopkMinBlocks) topk_rows_ker
                 int slot_i = pending + incl - c;
                 for (uint32_t b = hv; b; b &= b - 1) {
                     const int q = __ffs(b) - 1;
-                    uint32_t m = vector_hits<DT>(sk + v0 + q * 32 + lane, theta);
+                    uint32_t m = cell_hits<DT>(sk, v0 + q * 32 + lane, theta, cut, full_units);
                     while (m) {
                         const int i = __ffs(m) - 1;
                         m &= m - 1;
@@ -1342,7 +1404,8 @@ cudaError_t launch_dtype(const RowStatsArgs &a, int grid, int topk_grid, cudaStr
     st.k = 0;
     cudaError_t e = launch_typed<DT, true>(st, grid, stream);
     if (e != cudaSuccess) return e;
-    return launch_pdl(topk_rows_kernel<DT>, dim3(topk_grid), dim3(kTopkWarps * 32), 0, stream, a);
+    return a.few_chunks ? launch_pdl(topk_rows_kernel<DT, true>, dim3(topk_grid), dim3(kTopkWarps * 32), 0, stream, a)
+                        : launch_pdl(topk_rows_kernel<DT, false>, dim3(topk_grid), dim3(kTopkWarps * 32), 0, stream, a);
 }
 
 template <int DT>

@@ -41,6 +41,7 @@ __host__ __device__ constexpr int64_t sketch_entries(int64_t units) {
 #ifndef RPS_RING_STAGES
 #define RPS_RING_STAGES 2
 #endif
+constexpr int kFewChunks = 32;                   // ring chunks of a short row in the top-k launch
 constexpr int kBatch = RPS_RING_UNITS_PER_LANE;  // 16-byte units a lane takes from each ring buffer
 constexpr int kStages = RPS_RING_STAGES;         // ring buffers (bulk copies in flight) per warp
 
@@ -83,6 +84,7 @@ struct RowStatsArgs {
     int64_t units_per_row;
     int32_t warps;
     int64_t min_piece;    // at least ceil(units_per_row / (kMaxPartials - 1))
+    int32_t few_chunks;   // no cut leaves a row more than kFewChunks ring chunks (top-k mode)
     int32_t max_ppr;      // ceil(units_per_row / min_piece): pieces a row is cut into at most
     uint32_t *err;
 };

@@ -42,13 +42,15 @@ def test_cut(n, V, bf16, k):
     compare_stats(stats_np(out), oracle_default().row_stats(host[0, 0], k), np.arange(n), k, f"{n} x {V}")
 
 
-@pytest.mark.parametrize("k", [16, 17, 31, 32])
+@pytest.mark.parametrize("V", [40, 100, 3447, 7680, 7684, 32003])  # few chunks up to V 7,680; a cell a lane from 128
+@pytest.mark.parametrize("k", [10, 16, 17, 31, 32])
 @pytest.mark.parametrize("kind", ["spread", "equal", "few"])
-def test_long_lists(kind, k):
-    """The bound of long lists (two maxima per lane): spread rows, rows of equal
-    logits, and rows of fewer finite logits than k."""
-    rng = np.random.default_rng(k)
-    n, V = 9, 32003
+def test_lists(kind, k, V):
+    """The bound of the top-k search (one or two maxima per lane, over vectors of
+    cells or over the cells of short rows): spread rows, rows of equal logits, and
+    rows of fewer finite logits than k."""
+    rng = np.random.default_rng(k + V)
+    n = 9
     z = np.zeros((1, 1, n, V), np.float32)
     if kind == "spread":
         z[:] = rng.standard_normal(z.shape)
