@@ -922,6 +922,7 @@ cudaError_t launch_lm_k(int grid, cudaStream_t stream, const LmMaps &m, const Lm
     return a.kmax == 0    ? launch_lm<0, CG>(grid, stream, m, a)
            : a.kmax == 12 ? launch_lm<12, CG>(grid, stream, m, a)
            : a.kmax == 16 ? launch_lm<16, CG>(grid, stream, m, a)
+           : a.kmax == 20 ? launch_lm<20, CG>(grid, stream, m, a)
                           : launch_lm<32, CG>(grid, stream, m, a);
 }
 
@@ -965,7 +966,8 @@ rps_status lm_device(LmDevice *out) {
     LmDevice &d = g_lm_devices[dev];
     if (!d.ready) {
         if (cudaDeviceGetAttribute(&d.sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return RPS_ERR_CUDA;
-        if (set_smem<0>() != cudaSuccess || set_smem<12>() != cudaSuccess || set_smem<16>() != cudaSuccess || set_smem<32>() != cudaSuccess)
+        if (set_smem<0>() != cudaSuccess || set_smem<12>() != cudaSuccess || set_smem<16>() != cudaSuccess ||
+            set_smem<20>() != cudaSuccess || set_smem<32>() != cudaSuccess)
             return RPS_ERR_CUDA;
         if (count_pairs(&d.pairs) != cudaSuccess) return RPS_ERR_CUDA;
         d.ready = true;
@@ -1011,7 +1013,10 @@ rps_status make_packed_map(CUtensorMap *m, const void *base, int64_t blocks, int
     return encode(m, CU_TENSOR_MAP_DATA_TYPE_INT64, 3, base, dims, strides, box, false);
 }
 
-int list_len(int32_t k) { return k == 0 ? 0 : k <= 12 ? 12 : k <= 16 ? 16 : 32; }
+// Entries of the splits' lists. An insertion costs about as many instructions as
+// six times the length, and a CTA with one or two tiles little else: 100 rows of V
+// 32,000, d 1,024 at k = 20: 34.7 us with 20 entries, 41.5 with 32; k = 10: 12 for 16.
+int list_len(int32_t k) { return k == 0 ? 0 : k <= 12 ? 12 : k <= 16 ? 16 : k <= 20 ? 20 : 32; }
 
 struct LmLayout {
     size_t health, part, lists, total;
@@ -1155,6 +1160,7 @@ rps_status rps_lmhead_row_stats(const rps_lmhead *lm, const rps_params *prm, con
     if (a.kmax == 0) e = launch_pdl(lmhead_merge_kernel<0>, mgrid, dim3(kMergeThreads), 0, s, a);
     else if (a.kmax == 12) e = launch_pdl(lmhead_merge_kernel<12>, mgrid, dim3(kMergeThreads), 0, s, a);
     else if (a.kmax == 16) e = launch_pdl(lmhead_merge_kernel<16>, mgrid, dim3(kMergeThreads), 0, s, a);
+    else if (a.kmax == 20) e = launch_pdl(lmhead_merge_kernel<20>, mgrid, dim3(kMergeThreads), 0, s, a);
     else e = launch_pdl(lmhead_merge_kernel<32>, mgrid, dim3(kMergeThreads), 0, s, a);
     return e == cudaSuccess ? RPS_OK : RPS_ERR_CUDA;
 }

@@ -105,6 +105,8 @@ def test_lmhead_pairs(n, d, V, k):
     (1300, 9000, 20, 0),   # 13 splits for 20 ranks: the bound is taken two entries deep
     (5, 300, 32, 0),       # two splits: the bound at the lists' last entries
     (3, 20, 20, 0),        # one split, every token listed
+    (140, 5000, 16, 0),    # the list lengths in between
+    (140, 5000, 21, 0),
     (1, 33000, 12, 0),     # one row: a hidden copy of one row
     (4, 40000, 16, 2),     # two rows of equal logits: every list entry is a candidate
 ])
