@@ -338,6 +338,26 @@ __device__ __forceinline__ void list_insert(RowState<KMAX> &st, float z, int id)
     st.li[0] = z > top ? id : top_i;
 }
 
+// Sorts v descending (bitonic network over registers).
+template <int N>
+__device__ __forceinline__ void sort_desc(float (&v)[N]) {
+#pragma unroll
+    for (int size = 2; size <= N; size <<= 1) {
+#pragma unroll
+        for (int stride = size >> 1; stride > 0; stride >>= 1) {
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+                const int j = i ^ stride;
+                if (j > i) {
+                    const float hi = fmaxf(v[i], v[j]), lo = fminf(v[i], v[j]);
+                    v[i] = (i & size) == 0 ? hi : lo;
+                    v[j] = (i & size) == 0 ? lo : hi;
+                }
+            }
+        }
+    }
+}
+
 // The float below x (-inf and NaN stay).
 __device__ __forceinline__ float next_below(float x) {
     if (!(x > -INFINITY)) return x;
@@ -544,7 +564,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             // of a list, the maxima of its groups of columns bound the row's k-th
             // logit from below (k groups each hold one at least that large), so
             // that few columns enter the list (see pass 2).
-            constexpr int kGroup = KMAX > 16 ? 8 : 16;  // at least KMAX groups in a whole tile
+            constexpr int kGroup = 8, kGroups = kTileN / kGroup;  // 32: at least KMAX, and more bound closer
             float tm = -INFINITY;
             int ta = INT_MAX;
             for (int ch = 0; ch < n_ch; ++ch) {
@@ -559,24 +579,25 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
                 }
                 if (KMAX > 0 && t == 0) {
-#pragma unroll 1
-                    for (int g = 0; g < 32; g += kGroup) {
+#pragma unroll
+                    for (int g = 0; g < 32 / kGroup; ++g) {
                         float gm = -INFINITY;
 #pragma unroll
-                        for (int i = 0; i < 32; ++i)
-                            if (i / kGroup * kGroup == g && ch * 32 + i < ncol) gm = fmaxf(gm, v[i]);
-                        list_insert<KMAX>(st, gm, INT_MAX);
+                        for (int i = g * kGroup; i < (g + 1) * kGroup; ++i)
+                            if (ch * 32 + i < ncol) gm = fmaxf(gm, v[i]);
+                        pick[(ch * (32 / kGroup) + g) * (kEpiWarps * 32)] = gm;
                     }
                 }
             }
             if (KMAX > 0 && t == 0) {
+                float gm[kGroups];
+#pragma unroll
+                for (int g = 0; g < kGroups; ++g)
+                    gm[g] = g < n_ch * (32 / kGroup) ? pick[g * (kEpiWarps * 32)] : -INFINITY;
+                sort_desc(gm);
                 float kth = -INFINITY;
 #pragma unroll
-                for (int i = 0; i < (KMAX > 0 ? KMAX : 1); ++i) {
-                    kth = fmaxf(kth, i >= a.k - 1 ? st.lv[i] : -INFINITY);  // (sorted: entry k - 1)
-                    st.lv[i] = -INFINITY;
-                    st.li[i] = INT_MAX;
-                }
+                for (int g = 0; g < kGroups; ++g) kth = fmaxf(kth, g >= a.k - 1 ? gm[g] : -INFINITY);  // (entry k - 1)
                 floor_thr = next_below(kth);
             }
             if (tm > st.mx) {
