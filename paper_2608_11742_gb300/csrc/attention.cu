@@ -25,9 +25,9 @@
 //   warp 1      MMA issuer: S = Q K^T (M 128, N 128, K 128) into TMEM buffer t % 2 and
 //               O[t % 2] += P V^T, P read from TMEM, in one thread and in the
 //               order PV(t), S(t + 2), PV(t + 1), ...: the tensor pipe runs them in
-//               order, so S may overwrite the P just read with no wait, and one
-//               commit per tile stands for all they free. It also allocates and
-//               frees TMEM;
+//               order, so S may overwrite the P just read with no wait, and the
+//               commit of S(t + 2) stands for all that PV(t) frees but V. It also
+//               allocates and frees TMEM;
 //   warps 4-7   softmax of even tiles, warps 8-11 of odd ones: thread = query
 //               row, its 128 scores in registers (these warps take registers
 //               from the others with setmaxnreg). The base-2 reference m is
@@ -38,10 +38,10 @@
 //   warps 12-15 read-out: at the end of an item the halves' accumulators are
 //               weighted by 2^(m_half - m) / l, added and written as bf16, while the
 //               softmax goes on with the next item.
-// Bound by the MMA issue: the 16 instructions of a key tile and their commit take
+// Bound by the MMA issue: the 16 instructions of a key tile and a commit take
 // about 1,250 cycles back to back (1,024 of work), a tile about 2,100 with the
 // waits at the items' ends and for K and V; the softmax of a tile takes 1,500,
-// two run at once. 8 x 32 heads, context 512, 9 branches of 256: 266 -> 256 us;
+// two run at once. 8 x 32 heads, context 512, 9 branches of 256: 266 -> 254 us;
 // 32 heads, context 328, 9 branches of 32: 20.4 -> 14.7 us (against two halves
 // of each row in turn with separate S and P V issuers, and a tile per branch).
 // Every wait is bounded; a role whose wait runs out flags RPS_DEVERR_TIMEOUT
@@ -379,13 +379,16 @@ __device__ __forceinline__ void next_tile(int &n, int &j, int T) {
 }
 
 struct Ctl {
-    // One commit per tile, after S of tile t + 2, which follows the product of tile t in
+    // A commit per tile after S of tile t + 2, which follows the product of tile t in
     // the tensor pipe. s_full[t % 2]: S of tile t is computed and the product of
-    // tile t - 2 is done, so K stage t % 2, V stage t % 2 (of tile t - 2) and Q of
-    // the items before t's are free. No wait sees a barrier two phases on: each
+    // tile t - 2 is done, so K stage t % 2 and Q of the items before t's are free.
+    // V stage t % 2 has a commit of its own right after the product (v_empty):
+    // its next tile is then on its way while S of tile t + 2 is computed, which
+    // is worth more than the commit's 50 cycles (8 x 32 heads, context 512, 9
+    // branches of 256: 258 -> 254 us). No wait sees a barrier two phases on: each
     // waits for every phase in turn. (The read-out waits once an item, on a
     // barrier of its own: o_ready.)
-    uint64_t q_full[kQBufs], k_full[kKvStages], v_full[kKvStages];
+    uint64_t q_full[kQBufs], k_full[kKvStages], v_full[kKvStages], v_empty[kKvStages];
     uint64_t s_full[kHalves], p_full[kHalves], o_ready, o_free, mma_done;
     // a half's reference and sum of a row at the end of item n, in slot n % 4: it
     // is written before the half's last P of the item is handed on, read once
@@ -549,6 +552,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int s = 0; s < kKvStages; ++s) {
             mbar_init(&c.k_full[s], 1);
             mbar_init(&c.v_full[s], 1);
+            mbar_init(&c.v_empty[s], 1);
         }
         for (int b = 0; b < kHalves; ++b) {
             mbar_init(&c.s_full[b], 1);
@@ -619,11 +623,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     it = item_at(a, wk);
                 }
                 const int s = t % kKvStages;
-                // S of tile t is computed, so the product of tile t - 2 is done
-                // (phase 0 first: a barrier still in it would pass for phase 1 done)
-                if ((t >= kKvStages && t < 2 * kKvStages && !wait_or_abort(&c.s_full[s], 0, c, a)) ||
-                    (t >= kKvStages && !wait_or_abort(&c.s_full[s], (t / kKvStages) & 1, c, a)))
-                    break;
+                if (!wait_or_abort(&c.v_empty[s], ((t / kKvStages) & 1) ^ 1, c, a)) break;
                 int k0, valid;
                 key_tile(a, it, j, k0, valid);
                 uint8_t *dst = sv + s * kVBytes;
@@ -683,6 +683,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 for (int k = 0; k < 8; ++k)
                     mma_bf16_ts(ocol, pcol + k * 8, umma::advance_k16(k < 4 ? vd : vd1, k & 3), idesc,
                                 (j >= kHalves || k != 0) ? 1u : 0u, issue);
+                mma_commit(&c.v_empty[t % kKvStages], issue);
                 if (j == T - 1) mma_commit(&c.o_ready, issue);  // the item's O is complete
                 if (t + kHalves < tiles) ok = scores(t + kHalves);
             }
