@@ -57,7 +57,8 @@ FLUSH_BYTES = 256 << 20
 FALLBACK_HBM_GBS = 6800.0
 FALLBACK_BF16_TFLOPS = 1900.0
 LMHEAD_D = 4096  # hidden size of the 126,464-token model
-KERNEL_SOURCES = ("paper_2608_11742_gb300/csrc/rowstats.cu", "paper_2608_11742_gb300/csrc/rps_internal.cuh")
+KERNEL_SOURCES = ("paper_2608_11742_gb300/csrc/rowstats.cu", "paper_2608_11742_gb300/csrc/rps_internal.cuh",
+                  "paper_2608_11742_gb300/csrc/topk_device.cuh")
 
 
 class L2Flush:

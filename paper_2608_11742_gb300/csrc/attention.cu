@@ -38,12 +38,15 @@
 //   warps 12-15 read-out: at the end of an item the halves' accumulators are
 //               weighted by 2^(m_half - m) / l, added and written as bf16, while the
 //               softmax goes on with the next item.
-// Bound by the MMA issue: the 16 instructions of a key tile and a commit take
-// about 1,250 cycles back to back (1,024 of work), a tile about 2,100 with the
-// waits at the items' ends and for K and V; the softmax of a tile takes 1,500,
-// two run at once. 8 x 32 heads, context 512, 9 branches of 256: 266 -> 254 us;
-// 32 heads, context 328, 9 branches of 32: 20.4 -> 14.7 us (against two halves
-// of each row in turn with separate S and P V issuers, and a tile per branch).
+// Bound by the MMA issue: the 16 instructions of a key tile take 1,024 cycles of
+// work, and each commit costs their thread about 200 that instructions of N 128
+// do not hide: about 1,490 of the 2,050 cycles of a tile; the rest are its waits
+// (K, V, P, and the read-out at the items' ends). A half waits for S most of the
+// time: its softmax takes 1,330 to 1,540 cycles, and two run at once. Shared-memory
+// traffic is not the limit: pairs of CTAs that share K and V (160 -> 96 KB per tile)
+// took the same time. 8 x 32 heads, context 512, 9 branches of 256: 266 -> 254 us; 32
+// heads, context 328, 9 branches of 32: 20.4 -> 14.7 us (against two halves of each
+// row in turn with separate S and P V issuers, and a tile per branch).
 // Every wait is bounded; a role whose wait runs out flags RPS_DEVERR_TIMEOUT
 // and raises the CTA's abort flag, copies and MMAs in flight are drained and
 // TMEM is freed before the CTA exits.

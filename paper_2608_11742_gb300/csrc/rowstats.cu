@@ -5,9 +5,9 @@
 //   in top-k mode, T_i, mu_i and the truncated entropy of Eq. 3.
 //
 // Work split. One block of kStatThreads per SM; each warp streams one piece. With
-// at least as many warps as rows, each row is cut into equal pieces, so that no
-// piece crosses a row boundary (spread over the blocks when the rows are few);
-// otherwise the rows' 16-byte units are laid end to end and cut into equal
+// at least as many warps as rows, each row is mostly cut into equal pieces, so that
+// no piece crosses a row boundary (spread over the blocks when the rows are few;
+// piece_units has the rule); otherwise the rows' 16-byte units are laid end to end and cut into equal
 // contiguous pieces (a piece covers the tail of one row, whole rows and the head
 // of another). Either way every warp streams about the same number of bytes.
 // Each (warp, row) pair leaves a partial record in the

@@ -22,7 +22,8 @@ pytestmark = pytest.mark.gpu
     (1, 40001, True),      # 30 pieces, the last one short and ragged
     (162, 33000, True),    # as many pieces as fit: 30 a row, spread
     (163, 33000, True),    # 29 a row, neighbouring pieces together
-    (700, 9000, False),    # 6 a row leaves more than an eighth of the warps: the even cut
+    (700, 9000, False),    # 6 short pieces a row, though more than an eighth of the warps go idle
+    (1000, 45000, True),   # 4 long pieces a row would idle as many: the even cut, across rows
 ])
 @pytest.mark.parametrize("k", [0, 10])
 def test_cut(n, V, bf16, k):
