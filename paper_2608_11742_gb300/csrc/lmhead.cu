@@ -75,7 +75,10 @@ struct Shape {
     static constexpr int stage_bytes = slices * (kABytes + kBBytes / CG);
     // the ring, 32 logits per epilogue thread, and slack to align the ring to 1024 bytes
     static constexpr int smem_bytes = stages * stage_bytes + kEpiWarps * 32 * 32 * 4 + 1024;
-    static constexpr int granule = CG == 1 ? kTileN : kTileN / 2;   // tokens the splits are cut at
+    // Tokens the splits are cut at. Cut at whole tiles, the longest range of V
+    // 126,464 over 152 CTAs was four tiles against 3.25 on average, of V 44,273 two
+    // against 1.14: 32 rows, d 4,096 181 -> 172 us; 80 rows of V 44,273, d 1,216 47 -> 40.
+    static constexpr int granule = CG == 1 ? kTileN / 4 : kTileN / 2;
     static_assert(stages <= kMaxStages, "");
 };
 constexpr int kThreads = 192;               // warp 0 TMA, warp 1 MMA, warps 2-5 epilogue
@@ -442,7 +445,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             bool ok = true;
             for (int t = 0; t < n_tiles && ok; ++t) {
                 const int col0 = col_begin + t * kTileN;
-                const int n_cols = min(kTileN, col_end - col0);  // CG 2: 256, or 128 in a range's last tile
+                const int n_cols = min(kTileN, col_end - col0);  // 256, or whole granules in a range's last tile
                 for (int kb = 0; kb < kblocks; kb += Sh::slices) {
                     const int s = it % kStages;
                     const uint32_t ph = (it / kStages) & 1;
@@ -452,14 +455,23 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
                     uint8_t *sa = ring + s * kStageBytes;
                     if constexpr (CG == 1) {
-                        mbar_expect_tx(&c.full[s], h_bytes + kBBytes);
+                        mbar_expect_tx(&c.full[s], h_bytes + n_cols * kTileK * 2);
                         tma_load_2d(sa, &tm_h, kb * kTileK, row0, &c.full[s]);
-                        if (a.w_packed)  // one contiguous 32 KB block, already in the swizzled image
-                            bulk_load(sa + kABytes,
-                                      a.w_packed + (static_cast<int64_t>(col0 / kTileN) * kblocks + kb) * kBBytes, kBBytes,
-                                      &c.full[s]);
-                        else
-                            tma_load_2d(sa + kABytes, &tm_w, kb * kTileK, col0, &c.full[s]);
+                        uint8_t *sb = sa + kABytes;
+                        if (a.w_packed) {  // the rest of a 32 KB block, already in the swizzled image, and the next one's start
+                            const int off = col0 % kTileN, head = min(n_cols, kTileN - off);
+                            const uint8_t *blk =
+                                a.w_packed + (static_cast<int64_t>(col0 / kTileN) * kblocks + kb) * kBBytes;
+                            bulk_load(sb, blk + off * (kTileK * 2), head * (kTileK * 2), &c.full[s]);
+                            if (head < n_cols)
+                                bulk_load(sb + head * (kTileK * 2), blk + static_cast<int64_t>(kblocks) * kBBytes,
+                                          (n_cols - head) * (kTileK * 2), &c.full[s]);
+                        } else if (n_cols == kTileN) {
+                            tma_load_2d(sb, &tm_w, kb * kTileK, col0, &c.full[s]);
+                        } else {  // (tm_w_half: a granule per copy)
+                            for (int g = 0; g < n_cols; g += Sh::granule)
+                                tma_load_2d(sb + g * (kTileK * 2), &tm_w_half, kb * kTileK, col0 + g, &c.full[s]);
+                        }
                     } else {
                         // both CTAs' copies complete on the leader's barrier, which
                         // expects the bytes of both
@@ -1043,9 +1055,15 @@ struct LmLayout {
     size_t health, part, lists, total;
 };
 
-LmLayout lm_layout(int32_t n_rows, int64_t vocab, int32_t k) {
-    const int64_t n_vt = (vocab + kTileN - 1) / kTileN;
-    const size_t cap = static_cast<size_t>(n_rows) * static_cast<size_t>(std::min<int64_t>(n_vt, kMaxSplits));
+// Splits the workspace is laid out for. One row tile takes every SM, also with
+// fewer vocabulary tiles than SMs.
+int64_t splits_cap(int32_t n_rows, int64_t vocab) {
+    const int tokens = n_rows <= kTileM ? Shape<1>::granule : kTileN;
+    return std::min<int64_t>((vocab + tokens - 1) / tokens, kMaxSplits);
+}
+
+LmLayout lm_layout(int32_t n_rows, int64_t splits, int32_t k) {
+    const size_t cap = static_cast<size_t>(n_rows) * static_cast<size_t>(splits);
     auto up = [](size_t x) { return (x + 255) / 256 * 256; };
     LmLayout l;
     l.health = 0;
@@ -1082,7 +1100,7 @@ rps_status rps_lmhead_pack_unembed(const void *unembed, int64_t vocab, int32_t d
 
 size_t rps_lmhead_workspace_bytes(int32_t n_rows, int64_t vocab, int32_t k_max) {
     if (n_rows < 1 || vocab < 1 || vocab > INT32_MAX || k_max < 0 || k_max > RPS_MAX_K) return 0;
-    return lm_layout(n_rows, vocab, k_max).total;
+    return lm_layout(n_rows, splits_cap(n_rows, vocab), k_max).total;
 }
 
 rps_status rps_lmhead_row_stats(const rps_lmhead *lm, const rps_params *prm, const rps_row_stats *out,
@@ -1102,7 +1120,12 @@ rps_status rps_lmhead_row_stats(const rps_lmhead *lm, const rps_params *prm, con
         if (prm->k_max > lm->vocab || !out->topk_logit || !out->mu || !out->htrunc) return RPS_ERR_INVALID_ARG;
         k = prm->k_max;
     }
-    const LmLayout w = lm_layout(lm->n_rows, lm->vocab, k);
+    // The least workspace has room for a split per vocabulary tile; with less than
+    // the queried size there are no more splits than that.
+    const int n_vt = static_cast<int>((lm->vocab + kTileN - 1) / kTileN);
+    int64_t cap = splits_cap(lm->n_rows, lm->vocab);
+    if (ws_bytes < lm_layout(lm->n_rows, cap, k).total) cap = std::min(n_vt, kMaxSplits);
+    const LmLayout w = lm_layout(lm->n_rows, cap, k);
     if (!d_ws || ws_bytes < w.total || reinterpret_cast<uintptr_t>(d_ws) % 16) return RPS_ERR_INVALID_ARG;
     LmDevice dev;
     rps_status st = lm_device(&dev);
@@ -1111,7 +1134,6 @@ rps_status rps_lmhead_row_stats(const rps_lmhead *lm, const rps_params *prm, con
     if (!err) return RPS_ERR_CUDA;
 
     const int n_rt = (lm->n_rows + kTileM - 1) / kTileM;
-    const int n_vt = static_cast<int>((lm->vocab + kTileN - 1) / kTileN);
     // CTA pairs or single CTAs. A pair shares each unembedding tile, half in each
     // CTA: 32 KB per 64-wide slice and CTA instead of 48, from L2 and into shared
     // memory. An odd row tile makes a pair with an empty half, which costs as much
@@ -1124,7 +1146,13 @@ rps_status rps_lmhead_row_stats(const rps_lmhead *lm, const rps_params *prm, con
     const int64_t packed_blocks = static_cast<int64_t>(n_vt) * kblocks;
     const bool pair = (n_rt % 2 == 0 || n_rt >= 7) && dev.pairs >= 1 && packed_blocks <= INT32_MAX;
     const int units = pair ? (n_rt + 1) / 2 : n_rt;  // pairs or CTAs per split
-    const int splits = std::max(1, std::min({(pair ? dev.pairs : dev.sm_count) / units, n_vt, kMaxSplits}));
+    const int granule = pair ? Shape<2>::granule : Shape<1>::granule;
+    const int n_gran = static_cast<int>((lm->vocab + granule - 1) / granule);
+    int splits = std::max(1, std::min((pair ? dev.pairs : dev.sm_count) / units, static_cast<int>(cap)));
+    const int longest = (n_gran + splits - 1) / splits;
+    // As few as keep the longest range as short: more only make merging work (V
+    // 40,115, 33 rows, d 3,904: 152 splits 69 us, 126 splits 63).
+    splits = (n_gran + longest - 1) / longest;
     LmMaps maps;
     std::memset(&maps, 0, sizeof maps);
     if (pair) {
@@ -1139,10 +1167,11 @@ rps_status rps_lmhead_row_stats(const rps_lmhead *lm, const rps_params *prm, con
     } else {
         st = make_map(&maps.h, lm->hidden, lm->n_rows, lm->d, lm->hidden_stride, std::min<int32_t>(lm->n_rows, kTileM));
         if (st != RPS_OK) return st;
-        maps.w = maps.h;  // (single CTAs read the packed unembedding without a tensor map)
-        if (!lm->unembed_packed &&
-            (st = make_map(&maps.w, lm->unembed, lm->vocab, lm->d, lm->unembed_stride, kTileN)) != RPS_OK)
-            return st;
+        maps.w = maps.w_half = maps.h;  // (single CTAs read the packed unembedding without a tensor map)
+        for (int part = 0; part < 2 && !lm->unembed_packed && st == RPS_OK; ++part)
+            st = make_map(part ? &maps.w_half : &maps.w, lm->unembed, lm->vocab, lm->d, lm->unembed_stride,
+                          part ? Shape<1>::granule : kTileN);
+        if (st != RPS_OK) return st;
     }
 
     LmArgs a;
@@ -1173,8 +1202,7 @@ rps_status rps_lmhead_row_stats(const rps_lmhead *lm, const rps_params *prm, con
     a.topk_logit = out->topk_logit;
 
     const cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    const int granule = pair ? Shape<2>::granule : Shape<1>::granule;
-    a.n_gran = static_cast<int>((lm->vocab + granule - 1) / granule);
+    a.n_gran = n_gran;
     cudaError_t e = pair ? launch_lm_k<2>(units * splits * 2, s, maps, a) : launch_lm_k<1>(units * splits, s, maps, a);
     if (e != cudaSuccess) return RPS_ERR_CUDA;
     const dim3 mgrid(std::min((lm->n_rows + kMergeThreads / 32 - 1) / (kMergeThreads / 32), dev.sm_count * 8));

@@ -117,6 +117,49 @@ def test_lmhead_merge_lists(n, V, k, zero):
 
 
 @pytest.mark.parametrize("n,d,V,k", [
+    (7, 64, 68, 10),         # two granules, four tokens in the last, one K slice
+    (100, 320, 9800, 20),    # ranges of two granules (half a tile)
+    (33, 192, 40116, 0),     # ranges of five: a tile over two packed blocks, and one granule
+    (128, 128, 60000, 10),   # ranges of seven: a tile and three granules
+    (300, 64, 20004, 10),    # three row tiles of single CTAs
+])
+def test_lmhead_ranges(n, d, V, k):
+    """Vocabulary ranges of whole 64-token granules, row-major and packed alike; a workspace of
+    the least size accepted (a split per vocabulary tile) works, one of a byte less is refused."""
+    h, w = synth.lmhead_inputs(23, n, V, d)
+    rows = np.unique(np.linspace(0, n - 1, 24).astype(int))
+    check(h, w, k, rows=rows)
+    out, lg, ws = run_lmhead(h, w, k)
+    hd, wd = dev_bf16(h), dev_bf16(w)
+    packed = rps.RowStatsBuf.alloc(n, k, "cuda")
+    lp = torch.empty_like(lg)
+    pw = rps.rps_lmhead_pack_unembed(wd)
+    rps.rps_lmhead_row_stats(hd, wd, Prm(k) if k else None, packed, ws, lp, packed=pw)
+    assert rps.rps_poll_device_status() == (rps.RPS_OK, 0)
+    fields = ("zmax", "lse", "H", "pmax", "argmax") + (("mu", "htrunc", "topk_idx", "topk_logit") if k else ())
+    assert torch.equal(lg, lp)
+    for f in fields:
+        assert torch.equal(getattr(out, f), getattr(packed, f)), f
+    cap = n * ((V + 255) // 256)
+    up = lambda x: (x + 255) // 256 * 256
+    least = 256 + up(cap * 32) + up(cap * 8 * (0 if k == 0 else 12 if k <= 12 else 20))
+    small = ws[:least]
+    rps.rps_workspace_init(small)
+    few = rps.RowStatsBuf.alloc(n, k, "cuda")
+    rps.rps_lmhead_row_stats(hd, wd, Prm(k) if k else None, few, small, lp, packed=pw)
+    assert rps.rps_poll_device_status() == (rps.RPS_OK, 0)
+    assert torch.equal(lg, lp)
+    o = oracle_default().row_stats(lg.cpu().numpy()[rows], k)
+    g = stats_np(few)
+    for name in ("zmax", "lse", "H", "pmax") + (("mu", "htrunc") if k else ()):
+        assert_close(getattr(g, name)[rows], getattr(o, name), name)
+    for f in ("argmax",) + (("topk_idx", "topk_logit") if k else ()):
+        assert torch.equal(getattr(out, f), getattr(few, f)), f
+    with pytest.raises(rps.RPSError):
+        rps.rps_lmhead_row_stats(hd, wd, Prm(k) if k else None, few, small[:-1], None, packed=pw)
+
+
+@pytest.mark.parametrize("n,d,V,k", [
     (200, 128, 1000, 10),     # ragged rows and vocabulary, one tile per CTA
     (64, 64, 151936, 1),      # one K slice; the last vocabulary tile holds 128 tokens
     (130, 4096, 8192, 32),    # 64 K slices per tile, the longest list
