@@ -13,8 +13,9 @@
 // finding it in L2. Two row tiles can share a CTA pair (cta_group::2): M = 256
 // over both, half of each unembedding tile in either CTA.
 //   warp 0      TMA producer: per stage, the hidden tile's and the unembedding
-//               tile's 64-wide slices of d, 128-byte swizzle, into a ring of
-//               shared-memory stages (mbarrier completion, bounded waits). A
+//               tile's 64-wide slices of d (one, or several of a narrow
+//               tile), 128-byte swizzle, into a ring of shared-memory stages
+//               (mbarrier completion, bounded waits). A
 //               pair takes two slices per stage and one copy per operand: with
 //               a copy per 64 rows and slice the one issuing thread set the pace
 //               (512 rows: 329 us against 309);
@@ -64,7 +65,7 @@ constexpr int kMmaK = 16;                   // K of one tcgen05.mma kind::f16
 constexpr int kABytes = kTileM * kTileK * 2;  // 16 KB
 constexpr int kBBytes = kTileN * kTileK * 2;  // 32 KB
 constexpr int kEpiWarps = 4;
-constexpr int kMaxStages = 4;
+constexpr int kMaxStages = 5;
 constexpr int kLineRows = 16;               // packed rows (128 bytes each) per line of the pair's tensor map
 // Shape of the contraction by CTA group: one CTA (CG 1) with the whole
 // unembedding tile in its stages, or a pair (CG 2) with half of it each.
@@ -74,13 +75,24 @@ struct Shape {
     static constexpr int slices = CG == 1 ? 1 : 2;              // 64-wide slices of d per stage
     static constexpr int stage_bytes = slices * (kABytes + kBBytes / CG);
     // the ring, 32 logits per epilogue thread, and slack to align the ring to 1024 bytes
-    static constexpr int smem_bytes = stages * stage_bytes + kEpiWarps * 32 * 32 * 4 + 1024;
+    static constexpr int ring_bytes = stages * stage_bytes;
+    static constexpr int smem_bytes = ring_bytes + kEpiWarps * 32 * 32 * 4 + 1024;
     // Tokens the splits are cut at. Cut at whole tiles, the longest range of V
     // 126,464 over 152 CTAs was four tiles against 3.25 on average, of V 44,273 two
     // against 1.14: 32 rows, d 4,096 181 -> 172 us; 80 rows of V 44,273, d 1,216 47 -> 40.
     static constexpr int granule = CG == 1 ? kTileN / 4 : kTileN / 2;
     static_assert(stages <= kMaxStages, "");
 };
+// A single CTA's ring cut by its rows (FLEX): with few rows a fifth stage fits, and
+// a narrow last tile takes several slices of d per stage, since each stage costs
+// its barriers and commit whatever it holds. 32 rows of V 126,464, d 4,096 172 -> 164 us
+// (with the fifth stage alone 167); 53 rows of V 8,723, d 3,456 35 -> 31. Twelve stages of
+// one slice instead of four of three: 38.5.
+__host__ __device__ constexpr int slice_rows_bytes(int rows) { return (rows * kTileK * 2 + 1023) / 1024 * 1024; }  // (the swizzle's period)
+__host__ __device__ __forceinline__ int tile_slices(int n_cols, int a_bytes, int stage_bytes) {
+    const int n = stage_bytes / (a_bytes + n_cols * kTileK * 2);
+    return n < 4 ? n : 4;
+}
 constexpr int kThreads = 192;               // warp 0 TMA, warp 1 MMA, warps 2-5 epilogue
 constexpr uint32_t kTmemCols = 2 * kTileN;  // two accumulators
 constexpr int kMaxSplits = 256;
@@ -102,6 +114,7 @@ struct __align__(16) LmPartial {
 struct LmArgs {
     int32_t n_rows, d, n_gran, splits, kmax, k;  // n_gran: granules of the vocabulary
     int32_t h_rows;  // rows of a hidden copy: a tile's, or all of fewer
+    int32_t stages, stage_bytes;  // the ring (CG 1)
     const uint8_t *w_packed;  // unembedding in the packed tile layout, or nullptr (tensor map)
     int64_t vocab;
     LmPartial *part;   // [n_rows][splits]
@@ -369,13 +382,18 @@ __device__ __forceinline__ float next_below(float x) {
     return __uint_as_float(x > 0.f ? b - 1 : b + 1);
 }
 
-template <int KMAX, int CG>
+// FLEX: the ring cut by the launch's rows (CG 1)
+template <int KMAX, int CG, bool FLEX>
 __global__ void __launch_bounds__(kThreads, 1)
     lmhead_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_constant__ CUtensorMap tm_w,
                   const __grid_constant__ CUtensorMap tm_w_half, const LmArgs a) {
     using Sh = Shape<CG>;
-    constexpr int kStages = Sh::stages;
-    constexpr int kStageBytes = Sh::stage_bytes;
+    const int n_stages = FLEX ? a.stages : Sh::stages;
+    const int stage_bytes = FLEX ? a.stage_bytes : Sh::stage_bytes;
+    // Bytes of a slice's hidden tile in a stage. The MMA reads 16 KB from its start:
+    // what lies there beyond fewer rows (inside the dynamic shared memory: 16 KB
+    // follow the ring) are rows past the last, whose results nobody uses.
+    const int a_bytes = FLEX ? slice_rows_bytes(a.h_rows) : kABytes;
     extern __shared__ uint8_t dyn_smem[];
     __shared__ Ctl c;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -397,7 +415,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint8_t *ring = dyn_smem + ((1024u - (saddr(dyn_smem) & 1023u)) & 1023u);
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < kStages; ++s) {
+        for (int s = 0; s < n_stages; ++s) {
             mbar_init(&c.full[s], 1);
             mbar_init(&c.empty[s], 1);
         }
@@ -418,9 +436,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         tmem_relinquish<CG>();
     }
     if (CG == 2 && !has_rows) {
-        for (int i = threadIdx.x; i < kStages * Sh::slices * kABytes / 16; i += kThreads) {
+        for (int i = threadIdx.x; i < Sh::stages * Sh::slices * kABytes / 16; i += kThreads) {
             constexpr int kPerStage = Sh::slices * kABytes / 16;
-            *reinterpret_cast<uint4 *>(ring + i / kPerStage * kStageBytes + i % kPerStage * 16) = make_uint4(0, 0, 0, 0);
+            *reinterpret_cast<uint4 *>(ring + i / kPerStage * Sh::stage_bytes + i % kPerStage * 16) = make_uint4(0, 0, 0, 0);
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
@@ -440,38 +458,49 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (threadIdx.x == 0) flag_error(a.err, RPS_DEVERR_WORKSPACE);
     } else if (warp == 0) {
         if (lane == 0) {  // ---------------------------------------- TMA producer
+            uint32_t it = 0;  // stages filled
             const int pair_tiles = (rt | 1) * kTileM < a.n_rows ? 2 : 1;  // row tiles of the pair (CG 2)
-            uint32_t it = 0;
+            uint32_t ph = 0;
+            int s = 0;
             bool ok = true;
             for (int t = 0; t < n_tiles && ok; ++t) {
                 const int col0 = col_begin + t * kTileN;
                 const int n_cols = min(kTileN, col_end - col0);  // 256, or whole granules in a range's last tile
-                for (int kb = 0; kb < kblocks; kb += Sh::slices) {
-                    const int s = it % kStages;
-                    const uint32_t ph = (it / kStages) & 1;
+                const int slices = FLEX ? tile_slices(n_cols, a_bytes, stage_bytes) : Sh::slices;
+                // packed (CG 1): the rest of a 32 KB block, already in the swizzled
+                // image, and the start of the next tile's
+                const int off = col0 % kTileN, head = min(n_cols, kTileN - off);
+                const uint8_t *blk = a.w_packed + static_cast<int64_t>(col0 / kTileN) * kblocks * kBBytes +
+                                     static_cast<int64_t>(off) * kTileK * 2;
+                const int64_t next_blk = static_cast<int64_t>(kblocks) * kBBytes - static_cast<int64_t>(off) * kTileK * 2;
+                for (int kb = 0; kb < kblocks; kb += slices) {
                     if (!wait_or_abort(&c.empty[s], ph ^ 1, c, a)) {
                         ok = false;
                         break;
                     }
-                    uint8_t *sa = ring + s * kStageBytes;
+                    uint8_t *sa = ring + s * stage_bytes;
                     if constexpr (CG == 1) {
-                        mbar_expect_tx(&c.full[s], h_bytes + n_cols * kTileK * 2);
-                        tma_load_2d(sa, &tm_h, kb * kTileK, row0, &c.full[s]);
-                        uint8_t *sb = sa + kABytes;
-                        if (a.w_packed) {  // the rest of a 32 KB block, already in the swizzled image, and the next one's start
-                            const int off = col0 % kTileN, head = min(n_cols, kTileN - off);
-                            const uint8_t *blk =
-                                a.w_packed + (static_cast<int64_t>(col0 / kTileN) * kblocks + kb) * kBBytes;
-                            bulk_load(sb, blk + off * (kTileK * 2), head * (kTileK * 2), &c.full[s]);
-                            if (head < n_cols)
-                                bulk_load(sb + head * (kTileK * 2), blk + static_cast<int64_t>(kblocks) * kBBytes,
-                                          (n_cols - head) * (kTileK * 2), &c.full[s]);
-                        } else if (n_cols == kTileN) {
-                            tma_load_2d(sb, &tm_w, kb * kTileK, col0, &c.full[s]);
-                        } else {  // (tm_w_half: a granule per copy)
-                            for (int g = 0; g < n_cols; g += Sh::granule)
-                                tma_load_2d(sb + g * (kTileK * 2), &tm_w_half, kb * kTileK, col0 + g, &c.full[s]);
-                        }
+                        uint64_t *bar = &c.full[s];
+                        const int n_sl = min(slices, kblocks - kb);
+                        mbar_expect_tx(bar, n_sl * (h_bytes + n_cols * kTileK * 2));
+                        uint8_t *sb = sa + slices * a_bytes;
+                        int j = 0;
+                        do {
+                            tma_load_2d(sa, &tm_h, (kb + j) * kTileK, row0, bar);
+                            if (a.w_packed) {
+                                bulk_load(sb, blk, head * (kTileK * 2), bar);
+                                if (head < n_cols)
+                                    bulk_load(sb + head * (kTileK * 2), blk + next_blk, (n_cols - head) * (kTileK * 2), bar);
+                                blk += kBBytes;
+                            } else if (n_cols == kTileN) {
+                                tma_load_2d(sb, &tm_w, (kb + j) * kTileK, col0, bar);
+                            } else {  // (tm_w_half: a granule per copy)
+                                for (int g = 0; g < n_cols; g += Sh::granule)
+                                    tma_load_2d(sb + g * (kTileK * 2), &tm_w_half, (kb + j) * kTileK, col0 + g, bar);
+                            }
+                            sa += a_bytes;
+                            sb += n_cols * (kTileK * 2);
+                        } while (++j < n_sl);
                     } else {
                         // both CTAs' copies complete on the leader's barrier, which
                         // expects the bytes of both
@@ -491,18 +520,25 @@ __global__ void __launch_bounds__(kThreads, 1)
                             tma_load_3d_pair(sb, map, 0, tok, kb, bar);
                     }
                     ++it;
+                    if (++s == n_stages) {
+                        s = 0;
+                        ph ^= 1;
+                    }
                 }
             }
             // every copy issued lands before the CTA leaves, whichever role
             // aborted (in a normal run these phases have long completed). The
             // second CTA of a pair sees it by its stages being consumed.
-            for (uint32_t j = it > kStages ? it - kStages : 0; j < it; ++j)
-                wait_drain(rank == 0 ? &c.full[j % kStages] : &c.empty[j % kStages], (j / kStages) & 1);
+            const uint32_t ring_len = n_stages;
+            for (uint32_t j = it > ring_len ? it - ring_len : 0; j < it; ++j)
+                wait_drain(rank == 0 ? &c.full[j % ring_len] : &c.empty[j % ring_len], (j / ring_len) & 1);
         }
     } else if (warp == 1) {
         if (lane == 0 && rank == 0) {  // --------------------------- MMA issuer
-            uint32_t it = 0;
+            uint32_t ph = 0;
+            int s = 0;
             bool ok = true;
+            const uint64_t ring_desc = umma::smem_desc_kmajor_sw128(saddr(ring));
             for (int t = 0; t < n_tiles && ok; ++t) {
                 const int buf = t & 1;
                 const uint32_t use = static_cast<uint32_t>(t >> 1);
@@ -511,29 +547,34 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const uint32_t d_tmem = tmem + static_cast<uint32_t>(buf * kTileN);
                 const int n_cols = min(kTileN, col_end - (col_begin + t * kTileN));
                 const uint32_t idesc = umma::instr_desc_bf16(kTileM * CG, n_cols);
-                for (int kb = 0; kb < kblocks; kb += Sh::slices) {
-                    const int s = it % kStages;
-                    const uint32_t ph = (it / kStages) & 1;
+                const int slices = FLEX ? tile_slices(n_cols, a_bytes, stage_bytes) : Sh::slices;
+                const uint32_t a_step = a_bytes / 16, b_step = n_cols / CG * kTileK * 2 / 16, b_off = slices * a_step;
+                for (int kb = 0; kb < kblocks; kb += slices) {
                     if (!wait_or_abort(&c.full[s], ph, c, a)) {
                         ok = false;
                         break;
                     }
                     tc_fence_after();
+                    // (a descriptor's low bits are the address in 16-byte units)
+                    uint64_t ad = ring_desc + static_cast<uint32_t>(s * stage_bytes) / 16;
+                    uint64_t bd = ad + b_off;
+                    const auto slice_mmas = [&](bool first) {
 #pragma unroll
-                    for (int j = 0; j < Sh::slices; ++j) {
-                        if (j > 0 && kb + j >= kblocks) break;
-                        const uint32_t sa = saddr(ring + s * kStageBytes);
-                        const uint64_t ad = umma::smem_desc_kmajor_sw128(sa + j * kABytes);
-                        const uint64_t bd =
-                            umma::smem_desc_kmajor_sw128(sa + Sh::slices * kABytes + j * (n_cols / CG * kTileK * 2));
-#pragma unroll
-                        for (int k = 0; k < kTileK / kMmaK; ++k) {
+                        for (int k = 0; k < kTileK / kMmaK; ++k)
                             mma_bf16<CG>(d_tmem, umma::advance_k16(ad, k), umma::advance_k16(bd, k), idesc,
-                                         (kb | j | k) != 0 ? 1u : 0u);
-                        }
-                    }
+                                         k != 0 || !first ? 1u : 0u);
+                        ad += a_step;
+                        bd += b_step;
+                    };
+                    slice_mmas(kb == 0);
+                    if constexpr (FLEX)
+                        for (int j = 1; j < slices && kb + j < kblocks; ++j) slice_mmas(false);
+                    else if (Sh::slices > 1 && kb + 1 < kblocks) slice_mmas(false);
                     mma_commit<CG>(&c.empty[s]);  // the stage is free once these MMAs have read it
-                    ++it;
+                    if (++s == n_stages) {
+                        s = 0;
+                        ph ^= 1;
+                    }
                 }
                 if (ok) mma_commit<CG>(&c.acc_full[buf]);
             }
@@ -558,7 +599,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             st.li[i] = INT_MAX;
         }
         float floor_thr = -INFINITY;  // logits up to this never enter the list
-        float *pick = reinterpret_cast<float *>(ring + kStages * kStageBytes) + (warp - 2) * 32 + lane;
+        float *pick = reinterpret_cast<float *>(ring + Sh::ring_bytes) + (warp - 2) * 32 + lane;
         bool ok = true;
         for (int t = 0; t < n_tiles; ++t) {
             const int buf = t & 1;
@@ -942,29 +983,32 @@ void lm_config(cudaLaunchConfig_t *cfg, cudaLaunchAttribute (&attr)[2], dim3 gri
     cfg->numAttrs = CG == 1 ? 1 : 2;
 }
 
-template <int KMAX, int CG>
+template <int KMAX, int CG, bool FLEX>
 cudaError_t launch_lm(int grid, cudaStream_t stream, const LmMaps &m, const LmArgs &a) {
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[2];
     lm_config<CG>(&cfg, attr, dim3(grid), stream);
-    return cudaLaunchKernelEx(&cfg, lmhead_kernel<KMAX, CG>, m.h, m.w, m.w_half, a);
+    return cudaLaunchKernelEx(&cfg, lmhead_kernel<KMAX, CG, FLEX>, m.h, m.w, m.w_half, a);
 }
 
-template <int CG>
+template <int CG, bool FLEX>
 cudaError_t launch_lm_k(int grid, cudaStream_t stream, const LmMaps &m, const LmArgs &a) {
-    return a.kmax == 0    ? launch_lm<0, CG>(grid, stream, m, a)
-           : a.kmax == 12 ? launch_lm<12, CG>(grid, stream, m, a)
-           : a.kmax == 16 ? launch_lm<16, CG>(grid, stream, m, a)
-           : a.kmax == 20 ? launch_lm<20, CG>(grid, stream, m, a)
-                          : launch_lm<32, CG>(grid, stream, m, a);
+    return a.kmax == 0    ? launch_lm<0, CG, FLEX>(grid, stream, m, a)
+           : a.kmax == 12 ? launch_lm<12, CG, FLEX>(grid, stream, m, a)
+           : a.kmax == 16 ? launch_lm<16, CG, FLEX>(grid, stream, m, a)
+           : a.kmax == 20 ? launch_lm<20, CG, FLEX>(grid, stream, m, a)
+                          : launch_lm<32, CG, FLEX>(grid, stream, m, a);
 }
 
 template <int KMAX>
 cudaError_t set_smem() {
-    cudaError_t e = cudaFuncSetAttribute(lmhead_kernel<KMAX, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(lmhead_kernel<KMAX, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          Shape<1>::smem_bytes);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(lmhead_kernel<KMAX, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute(lmhead_kernel<KMAX, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 Shape<1>::smem_bytes);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(lmhead_kernel<KMAX, 2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  Shape<2>::smem_bytes);
     return e;
 }
@@ -976,7 +1020,7 @@ cudaError_t count_pairs(int *pairs) {
     lm_config<2>(&cfg, attr, dim3(2), nullptr);
     cfg.attrs = attr + 1;
     cfg.numAttrs = 1;
-    return cudaOccupancyMaxActiveClusters(pairs, lmhead_kernel<32, 2>, &cfg);
+    return cudaOccupancyMaxActiveClusters(pairs, lmhead_kernel<32, 2, false>, &cfg);
 }
 constexpr int kMaxDevices = 64;
 std::mutex g_lm_mutex;
@@ -1203,7 +1247,16 @@ rps_status rps_lmhead_row_stats(const rps_lmhead *lm, const rps_params *prm, con
 
     const cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     a.n_gran = n_gran;
-    cudaError_t e = pair ? launch_lm_k<2>(units * splits * 2, s, maps, a) : launch_lm_k<1>(units * splits, s, maps, a);
+    // A single CTA's ring by its rows (FLEX), where that gives a fifth stage or
+    // several slices in the last tile's stages; otherwise its code only costs (607
+    // rows of V 15,010, d 2,432: 38.2 us without, 39.6 with).
+    const int a_bytes = slice_rows_bytes(a.h_rows), last_cols = (longest * granule - 1) % kTileN + 1;
+    a.stage_bytes = longest * granule < kTileN ? Shape<1>::stage_bytes : a_bytes + kBBytes;
+    a.stages = std::min(kMaxStages, Shape<1>::ring_bytes / a.stage_bytes);
+    const bool flex = a.stages > Shape<1>::stages || tile_slices(last_cols, a_bytes, a.stage_bytes) > 1;
+    cudaError_t e = pair   ? launch_lm_k<2, false>(units * splits * 2, s, maps, a)
+                    : flex ? launch_lm_k<1, true>(units * splits, s, maps, a)
+                           : launch_lm_k<1, false>(units * splits, s, maps, a);
     if (e != cudaSuccess) return RPS_ERR_CUDA;
     const dim3 mgrid(std::min((lm->n_rows + kMergeThreads / 32 - 1) / (kMergeThreads / 32), dev.sm_count * 8));
     if (a.kmax == 0) e = launch_pdl(lmhead_merge_kernel<0>, mgrid, dim3(kMergeThreads), 0, s, a);

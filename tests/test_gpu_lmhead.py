@@ -121,6 +121,7 @@ def test_lmhead_merge_lists(n, V, k, zero):
     (100, 320, 9800, 20),    # ranges of two granules (half a tile)
     (33, 192, 40116, 0),     # ranges of five: a tile over two packed blocks, and one granule
     (128, 128, 60000, 10),   # ranges of seven: a tile and three granules
+    (20, 2112, 9000, 10),    # ranges of one granule: four slices of d per stage, one left over
     (300, 64, 20004, 10),    # three row tiles of single CTAs
 ])
 def test_lmhead_ranges(n, d, V, k):
