@@ -423,7 +423,9 @@ rps_status rps_lmhead_pack_unembed(const void *unembed, int64_t vocab, int32_t d
 /* Workspace bytes of rps_lmhead_row_stats (k_max 0 for statistics only); 0 for
  * invalid arguments. The workspace needs no zeroing before its first use
  * except its first 256 bytes (the health word of rps_workspace_init), so
- * rps_workspace_init on the whole workspace is the simple rule. */
+ * rps_workspace_init on the whole workspace is the simple rule. With up to 128
+ * rows the size is for a split of the vocabulary per 64 tokens (256 at most); a
+ * workspace for one per 256 tokens is accepted too, and takes fewer splits. */
 size_t rps_lmhead_workspace_bytes(int32_t n_rows, int64_t vocab, int32_t k_max);
 
 /*
