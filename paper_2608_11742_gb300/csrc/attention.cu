@@ -45,7 +45,7 @@
 // time: its softmax takes 1,330 to 1,540 cycles, and two run at once. Shared-memory
 // traffic is not the limit: pairs of CTAs that share K and V (160 -> 96 KB per tile)
 // took the same time. 8 x 32 heads, context 512, 9 branches of 256: 266 -> 254 us; 32
-// heads, context 328, 9 branches of 32: 20.4 -> 14.7 us (against two halves of each
+// heads, context 328, 9 branches of 32: 20.4 -> 13.9 us (against two halves of each
 // row in turn with separate S and P V issuers, and a tile per branch).
 // Every wait is bounded; a role whose wait runs out flags RPS_DEVERR_TIMEOUT
 // and raises the CTA's abort flag, copies and MMAs in flight are drained and
