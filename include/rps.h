@@ -277,9 +277,13 @@ rps_status rps_score_branches(const rps_logits *anchor_logits, int32_t anchor_br
 /*
  * Commit decision (Algorithm 1; Eq. 4). Per searched pivot j the best slot is
  * the argmax of score over its valid tokens and [MASK]; ties keep [MASK], then
- * the higher-ranked token. gain_j = score(best) - score([MASK]). The request
- * commits the pivot with the largest gain_j > 0 (lower position on ties) to
- * its best token, or abstains. out->mask_* receives M' minus the committed
+ * the higher-ranked token. These are ties of the computed fp32 scores: where a
+ * token's and [MASK]'s scores are equal in exact arithmetic (all rows of D_j the
+ * same in both branches) they may round apart, and the larger one wins. The two
+ * launches that score the rows may cut a row differently, by their row counts,
+ * and the two means add their rows in different orders.
+ * gain_j = score(best) - score([MASK]). The request commits the pivot with the
+ * largest gain_j > 0 (lower position on ties) to its best token, or abstains. out->mask_* receives M' minus the committed
  * pivot and may alias the mask arrays given to rps_select_pivots.
  */
 rps_status rps_commit(const rps_branch_scores *scores, int32_t n_req, int32_t L, const rps_pivots *piv,

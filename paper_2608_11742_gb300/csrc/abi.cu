@@ -223,13 +223,15 @@ rps_status prepare_row_stats(const rps_logits *logits, const rps_row_list *rows,
     a.warps = grid * (kStatThreads / 32);
     *topk_grid_out = static_cast<int>(std::min<int64_t>((max_rows + kTopkWarps - 1) / kTopkWarps,
                                                          static_cast<int64_t>(dev.sm_count) * 16));
-    // a piece shorter than one ring chunk would cost its record and its ticket
-    // for less than one copy's worth of row
-    a.min_piece = std::max<int64_t>((a.units_per_row + (kMaxPartials - 2) - 1) / (kMaxPartials - 2),
-                                    std::min<int64_t>(a.units_per_row, 32 * kBatch));
+    a.min_piece = (a.units_per_row + (kMaxPartials - 2) - 1) / (kMaxPartials - 2);
     a.max_ppr = static_cast<int32_t>((a.units_per_row + a.min_piece - 1) / a.min_piece);
-    // a row lies in at most max_ppr + 1 pieces, each of which may end in a partial chunk
-    a.few_chunks = a.units_per_row / (32 * kBatch) + a.max_ppr + 1 <= kFewChunks;
+    // The ring chunks of a row under any cut, whose n parts are at most one more
+    // than the pieces of its length: one each while a piece fits a chunk, else at
+    // most the row's whole chunks and n.
+    const int64_t chunk = 32 * kBatch, longer = std::max<int64_t>(a.min_piece, chunk + 1);
+    const int64_t chunks = std::max<int64_t>(a.min_piece <= chunk ? a.max_ppr + 1 : 0,
+                                             a.units_per_row / chunk + (a.units_per_row + longer - 1) / longer + 1);
+    a.few_chunks = chunks <= kFewChunks;
     a.err = dev.err;
     *grid_out = grid;
     return RPS_OK;

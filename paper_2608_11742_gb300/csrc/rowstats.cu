@@ -5,12 +5,12 @@
 //   in top-k mode, T_i, mu_i and the truncated entropy of Eq. 3.
 //
 // Work split. One block of kStatThreads per SM; each warp streams one piece. With
-// at least as many warps as rows, each row is mostly cut into equal pieces, so that
-// no piece crosses a row boundary (spread over the blocks when the rows are few;
-// piece_units has the rule); otherwise the rows' 16-byte units are laid end to end and cut into equal
-// contiguous pieces (a piece covers the tail of one row, whole rows and the head
-// of another). Either way every warp streams about the same number of bytes.
-// Each (warp, row) pair leaves a partial record in the
+// at least as many warps as rows, each row is cut into equal pieces where that
+// keeps the warps busy, so that no piece crosses a row boundary; otherwise the
+// rows' 16-byte units are laid end to end and cut into equal contiguous pieces (a
+// piece covers the tail of one row, whole rows and the head of another; with few
+// rows a warp takes one part of one row). Either way every warp streams about
+// the same number of bytes. Each (piece, row) pair leaves a partial record in the
 // workspace and the last warp to finish a row (atomic ticket, no waiting) merges
 // the at most kMaxPartials records and writes the row.
 //
@@ -652,39 +652,39 @@ __device__ __forceinline__ int div_small(int a, int b) {
     return q;
 }
 
-// The cut of the rows' units into pieces, one per warp. Aligned: each row is
-// cut into `cpr` equal pieces (at most a.max_ppr), so that no piece crosses a
-// row boundary, where a warp's stream stops for the row's record. Taken when it
-// leaves at most an eighth of the warps idle, or when the rows are so few that
-// each is cut into max_ppr pieces (the even cut would then have pieces of the
-// same length, and as many idle warps), or when the pieces are short: then the
-// even cut's extra records cost more than the idle warps. bf16 rows, aligned
-// against even, us: V 9,807 1,000 rows 13.1 / 16.1, 4,000 rows 20.7 / 24.6; V 20,000
-// 1,000 rows 15.5 / 18.7, 4,000 rows 40.4 / 37.5; V 30,000 1,400 rows 22.2 / 24.3, 2,000
-// rows 37.0 / 31.6; V 45,000 700 rows 19.2 / 21.3, 1,400 rows 35.0 / 31.9; V 76,594 700
-// rows 30.9 / 29.2. Otherwise all units are cut evenly, in
-// pieces of at least min_piece units, and cpr is 0. few: each row is in max_ppr
-// pieces, and warps may be left over. Returns the units per piece.
+// The cut of the rows' units into pieces. Aligned: each row is cut into `cpr`
+// equal pieces (at most a.max_ppr), so that no piece crosses a row boundary,
+// where a warp's stream stops for the row's record; taken when it leaves at most
+// an eighth of the warps idle. Otherwise all units are cut evenly, in pieces of at
+// least min_piece units, and cpr is 0. few: the pieces are that short and warps
+// are left over, enough for one per part of a row.
+// The parts decide how a row's sums round, and scores that are equal in exact
+// arithmetic (a token and [MASK] over rows that are the same in their branches)
+// are told apart by that rounding. So this rule is part of the results: with
+// pieces of a ring chunk at least, or with the aligned cut also for rows of short
+// pieces (1,000 bf16 rows of V 9,807 16.1 -> 13.1 us), other slots win.
 __device__ __forceinline__ int64_t piece_units(const RowStatsArgs &a, int64_t total_rows, int64_t nv, int &cpr,
                                                bool &few) {
     cpr = 0;
     few = false;
-    if (total_rows <= a.warps && nv < (1 << 21) && a.warps < (1 << 21)) {
+    if (total_rows <= a.warps) {  // (rows, warps and units of a row fit 32 bits)
         const int rows = static_cast<int>(total_rows), n = static_cast<int>(nv);
-        const int per = div_small(a.warps, rows);
-        const int ppr = min(per, a.max_ppr);
-        const int piece = div_small(n + ppr - 1, ppr);
-        const int c = div_small(n + piece - 1, piece);
-        bool take = ppr == a.max_ppr || 8 * rows * c >= 7 * a.warps;
-        if (!take) {  // a piece times the units it is longer by than an even one, at most 330,000
-            const float w = static_cast<float>(a.warps), p = static_cast<float>(piece);
-            take = (p * w - static_cast<float>(rows) * static_cast<float>(n)) * p <= 330000.f * w;
+        int piece, c;
+        if (nv < (1 << 21)) {
+            const int ppr = min(div_small(a.warps, rows), a.max_ppr);
+            piece = div_small(n + ppr - 1, ppr);
+            c = div_small(n + piece - 1, piece);
+        } else {
+            const int ppr = min(a.warps / rows, a.max_ppr);
+            piece = (n + ppr - 1) / ppr;
+            c = (n + piece - 1) / piece;
         }
-        if (take) {
+        if (8 * rows * c >= 7 * a.warps) {  // (rows * c is at most the warps)
             cpr = c;
-            few = ppr == a.max_ppr;
             return piece;
         }
+        few = total_rows * nv <= (a.min_piece - 1) * a.warps && rows * (a.max_ppr + 1) <= a.warps;
+        if (few) return a.min_piece;
     }
     return max((total_rows * nv + a.warps - 1) / a.warps, a.min_piece);
 }
@@ -710,12 +710,6 @@ __device__ __forceinline__ SketchRow sketch_row(int len0, int piece, int full_un
     q.piece = piece;
     q.cps = (piece + kChunkUnits - 1) / kChunkUnits;
     return q;
-}
-
-// Segment 0 of row r under a cut of `piece` units per warp.
-__device__ __forceinline__ int sketch_len0(int64_t r, int64_t nv, int64_t piece, bool aligned) {
-    const int64_t off = aligned ? 0 : (r * nv) % piece;  // units of the first piece spent on earlier rows
-    return static_cast<int>(min(piece - off, nv));
 }
 
 // Sketch entry of the first chunk of the segment starting at unit u0.
@@ -830,35 +824,58 @@ __global__ void __launch_bounds__(kStatThreads, kStatBlocksPerSm) row_stats_kern
     const int64_t nv = a.units_per_row;
     const int64_t total = total_rows * nv;
     if (total == 0) return;
-    __shared__ int cut_cpr[kWarps];  // pieces per row of an aligned cut, 0 for the even cut
+    // Of a warp whose units lie in one row: the row's parts, its own number among
+    // them and the units of the first piece before the row. (Kept in shared memory,
+    // not live through the stream; no parts: a warp of the even cut.)
+    struct OneRow {
+        int parts, mine, before;
+    };
+    __shared__ OneRow one_row[kWarps];
     int cpr0;
     bool few;
     const int64_t piece = piece_units(a, total_rows, nv, cpr0, few);
-    const bool aligned = cpr0 > 0;
-    // With few rows the piece numbers go round the blocks, so that the pieces
-    // spread over every SM instead of filling the first blocks: 32 rows of
-    // 126,464 bf16 logits (960 pieces) held 30 of 152 SMs, which were bound by
-    // their issue slots, and the step of one such block took 56.2 us against
-    // 45.0 spread. With (nearly) all warps in use neighbouring pieces stay in
-    // one block: spread, the 256-position step was 1.2 % slower.
-    const int warp = few ? wib * static_cast<int>(gridDim.x) + static_cast<int>(blockIdx.x)
-                         : static_cast<int>(blockIdx.x) * kWarps + wib;
-    if (lane == 0) cut_cpr[wib] = cpr0;
     if (SKETCH && blockIdx.x == 0 && threadIdx.x == 0) *a.sketch_piece = static_cast<int>(min(piece, nv));
+    OneRow one{cpr0, 0, 0};
     Walk w0;
-    if (aligned) {  // (32-bit: piece and the pieces per row are below the row length)
+    if (cpr0 > 0) {  // (32-bit: piece and the pieces per row are below the row length)
+        const int warp = static_cast<int>(blockIdx.x) * kWarps + wib;
         const int row0 = div_small(warp, cpr0), part = warp - row0 * cpr0;
         if (row0 >= total_rows) return;
+        one.mine = part;
         w0.r = row0;
         w0.u = part * static_cast<int>(piece);
         w0.left = min(piece, nv - w0.u);
+    } else if (few) {
+        // The parts of few rows go round the blocks, so that they spread over every
+        // SM instead of filling the first blocks: 32 rows of 126,464 bf16 logits (960
+        // pieces) held 30 of 152 SMs, which were bound by their issue slots, and the
+        // step of one such block took 56.0 us against 43.9 spread. A piece that
+        // crosses a row boundary goes to two warps, one for each row's part:
+        // max_ppr + 1 places to a row. (With nearly all warps in use neighbouring
+        // pieces stay in one block: spread, the 256-position step was 1.2 % slower.)
+        const int w = wib * static_cast<int>(gridDim.x) + static_cast<int>(blockIdx.x);
+        const int places = a.max_ppr + 1, row0 = div_small(w, places), part = w - row0 * places;
+        if (row0 >= total_rows) return;
+        const int64_t begin = row0 * nv;
+        const int len = static_cast<int>(piece), n = static_cast<int>(nv);
+        one.before = begin < (1 << 22)
+                         ? static_cast<int>(begin) - div_small(static_cast<int>(begin), len) * len
+                         : static_cast<int>(begin % len);
+        const int from = max(part * len - one.before, 0), to = min((part + 1) * len - one.before, n);
+        if (from >= to) return;
+        one.mine = part;
+        one.parts = 1 + (n < (1 << 21) ? div_small(one.before + n - 1, len) : (one.before + n - 1) / len);
+        w0.r = row0;
+        w0.u = from;
+        w0.left = to - from;
     } else {
-        const int64_t g_begin = static_cast<int64_t>(warp) * piece;
+        const int64_t g_begin = (static_cast<int64_t>(blockIdx.x) * kWarps + wib) * piece;
         if (g_begin >= total) return;
         w0.r = g_begin / nv;
         w0.u = static_cast<int>(g_begin - w0.r * nv);
         w0.left = min(piece, total - g_begin);
     }
+    if (lane == 0) one_row[wib] = one;
     const int V = static_cast<int>(a.vocab);
     const int full_units = V / N;
 
@@ -918,6 +935,12 @@ __global__ void __launch_bounds__(kStatThreads, kStatBlocksPerSm) row_stats_kern
         issued = __shfl_sync(kFull, issued, 0);
     };
 
+    // Segment 0 of row r: the first piece without what it spends on earlier rows.
+    auto len0 = [&](int64_t r) -> int {
+        const volatile OneRow &o = one_row[wib];
+        const int64_t before = o.parts > 0 ? o.before : (r * nv) % piece;
+        return static_cast<int>(min(piece - before, nv));
+    };
     Walk walk = w0;
     int64_t r;
     Segment s;
@@ -931,10 +954,7 @@ __global__ void __launch_bounds__(kStatThreads, kStatBlocksPerSm) row_stats_kern
         typename E::Sketch *sketch =
             SKETCH ? static_cast<typename E::Sketch *>(a.sketch) + s.slot * a.sketch_stride : nullptr;
         const int cend = min(s.u1, full_units);
-        int key = SKETCH ? sketch_key(sketch_row(sketch_len0(r, nv, piece, aligned), static_cast<int>(min(piece, nv)),
-                                                 full_units),
-                                      s.u0)
-                         : 0;
+        int key = SKETCH ? sketch_key(sketch_row(len0(r), static_cast<int>(min(piece, nv)), full_units), s.u0) : 0;
         for (int cu = s.u0; cu < cend; cu += kChunkUnits) {
             int st;
             if (!acquire(st)) return;
@@ -967,24 +987,22 @@ __global__ void __launch_bounds__(kStatThreads, kStatBlocksPerSm) row_stats_kern
         unpack2(L.t, t_lo, t_hi);
         RowTotals rt = combine(L.mref, s_lo + s_hi, t_lo + t_hi, L.mx, am);
 
-        // the pieces (warps) that hold a part of row r
+        // the pieces that hold a part of row r, and this one's number among them
         int64_t w_first;
-        int count;
-        // (read back from shared memory so that it is not kept live through the stream)
-        const int cpr = *reinterpret_cast<volatile int *>(&cut_cpr[wib]);
-        if (cpr > 0) {
-            w_first = r * cpr;
-            count = cpr;
+        const int64_t warp = static_cast<int64_t>(blockIdx.x) * kWarps + wib;
+        int count = *reinterpret_cast<volatile int *>(&one_row[wib].parts);
+        if (count > 0) {
+            w_first = warp - *reinterpret_cast<volatile int *>(&one_row[wib].mine);
         } else {
             w_first = (r * nv) / piece;
             count = static_cast<int>(((r + 1) * nv - 1) / piece - w_first + 1);
         }
+        const int my = static_cast<int>(warp - w_first);
         const int64_t slot = s.slot;
         if (count == 1) {
-            write_row<SKETCH>(a, slot, rt, lane, SKETCH ? sketch_len0(r, nv, piece, aligned) : 0);
+            write_row<SKETCH>(a, slot, rt, lane, SKETCH ? len0(r) : 0);
             continue;
         }
-        const int my = static_cast<int>(warp - w_first);
         Partial *part = a.part + slot * kMaxPartials;
         if (lane == 0) {
             Partial p;
@@ -1026,7 +1044,7 @@ __global__ void __launch_bounds__(kStatThreads, kStatBlocksPerSm) row_stats_kern
             p.amax = __ldcg(&part[lane].amax);
         }
         rt = combine(p.mref, p.s, p.t, p.mx, p.amax);
-        write_row<SKETCH>(a, slot, rt, lane, SKETCH ? sketch_len0(r, nv, piece, aligned) : 0);
+        write_row<SKETCH>(a, slot, rt, lane, SKETCH ? len0(r) : 0);
     }
 }
 

@@ -1,7 +1,7 @@
 """The row statistics at the edges of the rows' cut into pieces: rows shorter than
-one ring chunk, one chunk, one more element; few rows (each in its largest number
-of pieces, spread over the blocks) and the row counts around which the cut
-changes form. Against the oracle, in both modes."""
+one ring chunk, one chunk, one more element; few rows (a warp per part of a row,
+spread over the blocks) and the row counts around which the cut changes form.
+Against the oracle, in both modes."""
 import numpy as np
 import pytest
 import torch
@@ -15,15 +15,15 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("n,V,bf16", [
     (1, 1, False),         # one piece of one value
-    (3, 1023, True),       # one unit short of a chunk, ragged
+    (3, 1023, True),       # a whole chunk's units less one value, in pieces of five units across rows
     (2, 1024, True),       # exactly one chunk
-    (5, 1025, True),       # one value more: two pieces
+    (5, 1025, True),       # one value more
     (7, 512 * 30, False),  # 30 pieces of one chunk
     (1, 40001, True),      # 30 pieces, the last one short and ragged
-    (162, 33000, True),    # as many pieces as fit: 30 a row, spread
-    (163, 33000, True),    # 29 a row, neighbouring pieces together
-    (700, 9000, False),    # 6 short pieces a row, though more than an eighth of the warps go idle
-    (1000, 45000, True),   # 4 long pieces a row would idle as many: the even cut, across rows
+    (162, 33000, True),    # 30 pieces a row, none across rows
+    (163, 33000, True),    # 29 a row
+    (700, 9000, False),    # 6 pieces a row would idle more than an eighth of the warps: the even cut, across rows
+    (1000, 45000, True),   # so would 4 long ones
 ])
 @pytest.mark.parametrize("k", [0, 10])
 def test_cut(n, V, bf16, k):
@@ -43,7 +43,7 @@ def test_cut(n, V, bf16, k):
     compare_stats(stats_np(out), oracle_default().row_stats(host[0, 0], k), np.arange(n), k, f"{n} x {V}")
 
 
-@pytest.mark.parametrize("V", [40, 100, 3447, 7680, 7684, 32003])  # few chunks up to V 7,680; a cell a lane from 128
+@pytest.mark.parametrize("V", [40, 100, 3447, 7680, 7684, 32003])  # few chunks up to V 8,188; a cell a lane from 128
 @pytest.mark.parametrize("k", [10, 16, 17, 31, 32])
 @pytest.mark.parametrize("kind", ["spread", "equal", "few"])
 def test_lists(kind, k, V):
