@@ -427,9 +427,11 @@ rps_status rps_lmhead_pack_unembed(const void *unembed, int64_t vocab, int32_t d
 /* Workspace bytes of rps_lmhead_row_stats (k_max 0 for statistics only); 0 for
  * invalid arguments. The workspace needs no zeroing before its first use
  * except its first 256 bytes (the health word of rps_workspace_init), so
- * rps_workspace_init on the whole workspace is the simple rule. With up to 128
- * rows the size is for a split of the vocabulary per 64 tokens (256 at most); a
- * workspace for one per 256 tokens is accepted too, and takes fewer splits. */
+ * rps_workspace_init on the whole workspace is the simple rule. The size does
+ * not fall as n_rows, vocab or k_max grow: a workspace queried for the largest
+ * call serves every smaller one. With up to 128 rows it is for a split of the
+ * vocabulary per 64 tokens (256 at most); a workspace for one per 256 tokens is
+ * accepted too, and takes fewer splits (the rows' sums then round differently). */
 size_t rps_lmhead_workspace_bytes(int32_t n_rows, int64_t vocab, int32_t k_max);
 
 /*

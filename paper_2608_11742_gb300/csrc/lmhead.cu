@@ -1144,7 +1144,11 @@ rps_status rps_lmhead_pack_unembed(const void *unembed, int64_t vocab, int32_t d
 
 size_t rps_lmhead_workspace_bytes(int32_t n_rows, int64_t vocab, int32_t k_max) {
     if (n_rows < 1 || vocab < 1 || vocab > INT32_MAX || k_max < 0 || k_max > RPS_MAX_K) return 0;
-    return lm_layout(n_rows, splits_cap(n_rows, vocab), k_max).total;
+    // one row tile may need more than a few rows of the next: a workspace queried for
+    // the largest row count has to do for every smaller one
+    size_t need = lm_layout(n_rows, splits_cap(n_rows, vocab), k_max).total;
+    if (n_rows > kTileM) need = std::max(need, lm_layout(kTileM, splits_cap(kTileM, vocab), k_max).total);
+    return need;
 }
 
 rps_status rps_lmhead_row_stats(const rps_lmhead *lm, const rps_params *prm, const rps_row_stats *out,

@@ -145,3 +145,13 @@ def test_host_rejects_bad_arguments(libs):
                                      C.c_uint32, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p]
     assert synth.rps_synth_fill(fake + 4, 1, 1, 8, 32, 4096, 0, 0, 4096, 0, 1, 2, 0, None, None, None, None) == 1
     assert synth.rps_synth_fill(fake, 1, 1, 8, 32, 4096, 0, 0, 4096, 0, 3, 2, 0, None, None, None, None) == 1
+
+
+@pytest.mark.parametrize("k", [0, 10, 20, 32])
+@pytest.mark.parametrize("vocab", [1, 300, 9000, 32000, 65600, 126464])
+def test_lmhead_workspace_does_not_fall_with_more_rows(libs, vocab, k):
+    """A workspace queried for the largest row count serves every smaller one in full."""
+    size = libs["librps.so"].rps_lmhead_workspace_bytes
+    size.restype, size.argtypes = C.c_size_t, [C.c_int32, C.c_int64, C.c_int32]
+    sizes = [size(n, vocab, k) for n in (1, 2, 64, 127, 128, 129, 200, 256, 257, 512, 1024, 4000)]
+    assert sizes[0] > 0 and sizes == sorted(sizes)
