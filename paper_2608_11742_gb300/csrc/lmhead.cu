@@ -51,6 +51,7 @@
 #include <cstring>
 #include <mutex>
 
+#include "lmhead_split.h"
 #include "rps_internal.cuh"
 #include "topk_device.cuh"
 #include "umma_desc.h"
@@ -58,8 +59,6 @@
 namespace rps {
 namespace {
 
-constexpr int kTileM = 128;                 // hidden rows per tile (TMEM lanes)
-constexpr int kTileN = 256;                 // tokens per tile (accumulator columns)
 constexpr int kTileK = 64;                  // d per stage: one 128-byte swizzle row of bf16
 constexpr int kMmaK = 16;                   // K of one tcgen05.mma kind::f16
 constexpr int kABytes = kTileM * kTileK * 2;  // 16 KB
@@ -77,10 +76,7 @@ struct Shape {
     // the ring, 32 logits per epilogue thread, and slack to align the ring to 1024 bytes
     static constexpr int ring_bytes = stages * stage_bytes;
     static constexpr int smem_bytes = ring_bytes + kEpiWarps * 32 * 32 * 4 + 1024;
-    // Tokens the splits are cut at. Cut at whole tiles, the longest range of V
-    // 126,464 over 152 CTAs was four tiles against 3.25 on average, of V 44,273 two
-    // against 1.14: 32 rows, d 4,096 181 -> 172 us; 80 rows of V 44,273, d 1,216 47 -> 40.
-    static constexpr int granule = CG == 1 ? kTileN / 4 : kTileN / 2;
+    static constexpr int granule = lm_granule(CG);  // tokens the splits are cut at
     static_assert(stages <= kMaxStages, "");
 };
 // A single CTA's ring cut by its rows (FLEX): with few rows a fifth stage fits, and
@@ -95,7 +91,6 @@ __host__ __device__ __forceinline__ int tile_slices(int n_cols, int a_bytes, int
 }
 constexpr int kThreads = 192;               // warp 0 TMA, warp 1 MMA, warps 2-5 epilogue
 constexpr uint32_t kTmemCols = 2 * kTileN;  // two accumulators
-constexpr int kMaxSplits = 256;
 constexpr int kMergeThreads = 128;
 constexpr uint64_t kDrainNs = 200ull * 1000 * 1000;
 constexpr float kLog2e = 1.4426950408889634f;
@@ -309,7 +304,6 @@ __device__ bool wait_or_abort(uint64_t *bar, uint32_t parity, Ctl &c, const LmAr
     return false;
 }
 
-// A wait that only ends early when the phase completes (drains before exit).
 // wait_or_abort for every lane of a warp that goes on to warp-wide tcgen05
 // instructions: the warp leaves together, on the same answer.
 template <typename Ctl_, typename Args_>
@@ -317,6 +311,7 @@ __device__ __forceinline__ bool warp_wait_or_abort(uint64_t *bar, uint32_t parit
     return __all_sync(kFull, wait_or_abort(bar, parity, c, a));
 }
 
+// A wait that only ends early when the phase completes (drains before exit).
 __device__ void wait_drain(uint64_t *bar, uint32_t parity) {
     if (mbar_try_wait(bar, parity)) return;
     const uint64_t start = global_ns();
@@ -1046,7 +1041,10 @@ rps_status lm_device(LmDevice *out) {
         if (set_smem<0>() != cudaSuccess || set_smem<12>() != cudaSuccess || set_smem<16>() != cudaSuccess ||
             set_smem<20>() != cudaSuccess || set_smem<32>() != cudaSuccess)
             return RPS_ERR_CUDA;
-        if (count_pairs(&d.pairs) != cudaSuccess) return RPS_ERR_CUDA;
+        int counted = 0;
+        const cudaError_t e = count_pairs(&counted);
+        if (e != cudaSuccess) cudaGetLastError();  // (not the next call's error)
+        d.pairs = lm_pairs(e == cudaSuccess, counted);
         d.ready = true;
     }
     *out = d;
@@ -1182,25 +1180,11 @@ rps_status rps_lmhead_row_stats(const rps_lmhead *lm, const rps_params *prm, con
     if (!err) return RPS_ERR_CUDA;
 
     const int n_rt = (lm->n_rows + kTileM - 1) / kTileM;
-    // CTA pairs or single CTAs. A pair shares each unembedding tile, half in each
-    // CTA: 32 KB per 64-wide slice and CTA instead of 48, from L2 and into shared
-    // memory. An odd row tile makes a pair with an empty half, which costs as much
-    // as two tiles: at 3 and 5 row tiles that is more than the pairs save. One row
-    // tile alone is bound by reading the unembedding. V 126,464, d 4,096, statistics
-    // only, single against pairs: 200 rows 232 / 189 us, 300 rows 271 / 292, 512 rows
-    // 338 / 309, 640 rows 442 / 447, 896 rows 605 / 586, 1,152 rows 765 / 734.
-    // (The packed unembedding's blocks are tensor coordinates in a pair, 32 bits.)
     const int kblocks = lm->d / kTileK;
     const int64_t packed_blocks = static_cast<int64_t>(n_vt) * kblocks;
-    const bool pair = (n_rt % 2 == 0 || n_rt >= 7) && dev.pairs >= 1 && packed_blocks <= INT32_MAX;
-    const int units = pair ? (n_rt + 1) / 2 : n_rt;  // pairs or CTAs per split
-    const int granule = pair ? Shape<2>::granule : Shape<1>::granule;
-    const int n_gran = static_cast<int>((lm->vocab + granule - 1) / granule);
-    int splits = std::max(1, std::min((pair ? dev.pairs : dev.sm_count) / units, static_cast<int>(cap)));
-    const int longest = (n_gran + splits - 1) / splits;
-    // As few as keep the longest range as short: more only make merging work (V
-    // 40,115, 33 rows, d 3,904: 152 splits 69 us, 126 splits 63).
-    splits = (n_gran + longest - 1) / longest;
+    const LmSplit sp = lm_split(n_rt, lm->vocab, packed_blocks, cap, dev.sm_count, dev.pairs);
+    const bool pair = sp.pair;
+    const int units = sp.units, granule = sp.granule, n_gran = sp.n_gran, splits = sp.splits, longest = sp.longest;
     LmMaps maps;
     std::memset(&maps, 0, sizeof maps);
     if (pair) {
