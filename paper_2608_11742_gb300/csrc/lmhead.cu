@@ -395,9 +395,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int rank = CG == 1 ? 0 : static_cast<int>(cluster_rank());
     const int unit = static_cast<int>(blockIdx.x) / CG;  // CTA or pair
     const int rt = unit / a.splits * CG + rank, split = unit % a.splits;
-    const int col_begin = static_cast<int>(static_cast<int64_t>(split) * a.n_gran / a.splits) * Sh::granule;
-    const int col_end = static_cast<int>(static_cast<int64_t>(split + 1) * a.n_gran / a.splits) * Sh::granule;
-    const int n_tiles = (col_end - col_begin + kTileN - 1) / kTileN;
+    const int col_begin = static_cast<int>(lm_range(split, a.n_gran, a.splits, Sh::granule));
+    const int64_t col_end = lm_range(split + 1, a.n_gran, a.splits, Sh::granule);
+    const int n_tiles = static_cast<int>((col_end - col_begin + kTileN - 1) / kTileN);
     const int kblocks = a.d / kTileK;
     // With fewer rows than a tile the hidden copies are that high: filling most of
     // a tile from outside so small a tensor is slow (V 126,464, d 4,096, k 10: 4 rows
@@ -460,7 +460,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             bool ok = true;
             for (int t = 0; t < n_tiles && ok; ++t) {
                 const int col0 = col_begin + t * kTileN;
-                const int n_cols = min(kTileN, col_end - col0);  // 256, or whole granules in a range's last tile
+                const int n_cols = static_cast<int>(min(static_cast<int64_t>(kTileN), col_end - col0));  // 256, or whole granules in a range's last tile
                 const int slices = FLEX ? tile_slices(n_cols, a_bytes, stage_bytes) : Sh::slices;
                 // packed (CG 1): the rest of a 32 KB block, already in the swizzled
                 // image, and the start of the next tile's
@@ -540,7 +540,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (!wait_or_abort(&c.acc_empty[buf], (use & 1) ^ 1, c, a)) break;
                 tc_fence_after();
                 const uint32_t d_tmem = tmem + static_cast<uint32_t>(buf * kTileN);
-                const int n_cols = min(kTileN, col_end - (col_begin + t * kTileN));
+                const int n_cols = static_cast<int>(min(static_cast<int64_t>(kTileN), col_end - (col_begin + t * kTileN)));
                 const uint32_t idesc = umma::instr_desc_bf16(kTileM * CG, n_cols);
                 const int slices = FLEX ? tile_slices(n_cols, a_bytes, stage_bytes) : Sh::slices;
                 const uint32_t a_step = a_bytes / 16, b_step = n_cols / CG * kTileK * 2 / 16, b_off = slices * a_step;
@@ -606,7 +606,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             tc_fence_after();
             const uint32_t tbase = tmem + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(buf * kTileN);
             const int col0 = col_begin + t * kTileN;
-            const int ncol = static_cast<int>(min(static_cast<int64_t>(min(kTileN, col_end - col0)), a.vocab - col0));
+            const int ncol = static_cast<int>(min(static_cast<int64_t>(kTileN), min(col_end, a.vocab) - col0));
             const int n_ch = (ncol + 31) / 32;
             // pass 1: the tile's maximum and its lowest column. In the first tile
             // of a list, the maxima of its groups of columns bound the row's k-th
@@ -1238,8 +1238,9 @@ rps_status rps_lmhead_row_stats(const rps_lmhead *lm, const rps_params *prm, con
     // A single CTA's ring by its rows (FLEX), where that gives a fifth stage or
     // several slices in the last tile's stages; otherwise its code only costs (607
     // rows of V 15,010, d 2,432: 38.2 us without, 39.6 with).
-    const int a_bytes = slice_rows_bytes(a.h_rows), last_cols = (longest * granule - 1) % kTileN + 1;
-    a.stage_bytes = longest * granule < kTileN ? Shape<1>::stage_bytes : a_bytes + kBBytes;
+    const int64_t range = static_cast<int64_t>(longest) * granule;  // of the longest split
+    const int a_bytes = slice_rows_bytes(a.h_rows), last_cols = static_cast<int>((range - 1) % kTileN) + 1;
+    a.stage_bytes = range < kTileN ? Shape<1>::stage_bytes : a_bytes + kBBytes;
     a.stages = std::min(kMaxStages, Shape<1>::ring_bytes / a.stage_bytes);
     const bool flex = a.stages > Shape<1>::stages || tile_slices(last_cols, a_bytes, a.stage_bytes) > 1;
     cudaError_t e = pair   ? launch_lm_k<2, false>(units * splits * 2, s, maps, a)

@@ -6,6 +6,12 @@
 #include <climits>
 #include <cstdint>
 
+#ifdef __CUDACC__
+#define LMSPLIT_HD __host__ __device__
+#else
+#define LMSPLIT_HD
+#endif
+
 namespace rps {
 
 constexpr int kTileM = 128;                 // hidden rows per tile (TMEM lanes)
@@ -51,6 +57,12 @@ inline LmSplit lm_split(int n_row_tiles, int64_t vocab, int64_t packed_blocks, i
     // 40,115, 33 rows, d 3,904: 152 splits 69 us, 126 splits 63).
     s.splits = (s.n_gran + s.longest - 1) / s.longest;
     return s;
+}
+
+// First token of a split's range (of the split after it: its end). Whole granules,
+// so the last range's end may lie past INT32_MAX.
+LMSPLIT_HD inline int64_t lm_range(int split, int n_gran, int splits, int granule) {
+    return static_cast<int64_t>(split) * n_gran / splits * granule;
 }
 
 }  // namespace rps
