@@ -65,6 +65,7 @@ constexpr int kABytes = kTileM * kTileK * 2;  // 16 KB
 constexpr int kBBytes = kTileN * kTileK * 2;  // 32 KB
 constexpr int kEpiWarps = 4;
 constexpr int kMaxStages = 5;
+constexpr int kCopyRows = kTileN / 4;       // unembedding rows per copy of a narrow tile (single CTAs)
 constexpr int kLineRows = 16;               // packed rows (128 bytes each) per line of the pair's tensor map
 // Shape of the contraction by CTA group: one CTA (CG 1) with the whole
 // unembedding tile in its stages, or a pair (CG 2) with half of it each.
@@ -76,7 +77,6 @@ struct Shape {
     // the ring, 32 logits per epilogue thread, and slack to align the ring to 1024 bytes
     static constexpr int ring_bytes = stages * stage_bytes;
     static constexpr int smem_bytes = ring_bytes + kEpiWarps * 32 * 32 * 4 + 1024;
-    static constexpr int granule = lm_granule(CG);  // tokens the splits are cut at
     static_assert(stages <= kMaxStages, "");
 };
 // A single CTA's ring cut by its rows (FLEX): with few rows a fifth stage fits, and
@@ -107,7 +107,8 @@ struct __align__(16) LmPartial {
 };
 
 struct LmArgs {
-    int32_t n_rows, d, n_gran, splits, kmax, k;  // n_gran: granules of the vocabulary
+    int32_t n_rows, d, splits, kmax, k;
+    int32_t granule, n_gran;  // tokens the splits are cut at, granules of the vocabulary
     int32_t h_rows;  // rows of a hidden copy: a tile's, or all of fewer
     int32_t stages, stage_bytes;  // the ring (CG 1)
     const uint8_t *w_packed;  // unembedding in the packed tile layout, or nullptr (tensor map)
@@ -134,16 +135,26 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
 __device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(saddr(bar)), "r"(bytes) : "memory");
 }
-// (cluster scope: the arrival may come from the pair's other CTA)
+// (a pair: cluster scope, the arrival may come from the other CTA)
+template <int CG>
 __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
     uint32_t done;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(done)
-        : "r"(saddr(bar)), "r"(parity)
-        : "memory");
+    if constexpr (CG == 1)
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(done)
+            : "r"(saddr(bar)), "r"(parity)
+            : "memory");
+    else
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(done)
+            : "r"(saddr(bar)), "r"(parity)
+            : "memory");
     return done != 0;
 }
 __device__ __forceinline__ uint64_t global_ns() {
@@ -290,11 +301,12 @@ struct Ctl {
 // Waits for phase `parity` of `bar`. False when the CTA aborts: this wait ran
 // out (then it flags the timeout, marks the workspace and raises the abort
 // flag) or another role already aborted.
+template <int CG>
 __device__ bool wait_or_abort(uint64_t *bar, uint32_t parity, Ctl &c, const LmArgs &a) {
-    if (a.wait_ns != 0 && mbar_try_wait(bar, parity)) return true;
+    if (a.wait_ns != 0 && mbar_try_wait<CG>(bar, parity)) return true;
     const uint64_t start = global_ns();
     while (a.wait_ns != 0) {
-        if (mbar_try_wait(bar, parity)) return true;
+        if (mbar_try_wait<CG>(bar, parity)) return true;
         if (*reinterpret_cast<volatile int *>(&c.abort_flag)) return false;
         if (global_ns() - start > a.wait_ns) break;
     }
@@ -306,17 +318,18 @@ __device__ bool wait_or_abort(uint64_t *bar, uint32_t parity, Ctl &c, const LmAr
 
 // wait_or_abort for every lane of a warp that goes on to warp-wide tcgen05
 // instructions: the warp leaves together, on the same answer.
-template <typename Ctl_, typename Args_>
+template <int CG, typename Ctl_, typename Args_>
 __device__ __forceinline__ bool warp_wait_or_abort(uint64_t *bar, uint32_t parity, Ctl_ &c, const Args_ &a) {
-    return __all_sync(kFull, wait_or_abort(bar, parity, c, a));
+    return __all_sync(kFull, wait_or_abort<CG>(bar, parity, c, a));
 }
 
 // A wait that only ends early when the phase completes (drains before exit).
+template <int CG>
 __device__ void wait_drain(uint64_t *bar, uint32_t parity) {
-    if (mbar_try_wait(bar, parity)) return;
+    if (mbar_try_wait<CG>(bar, parity)) return;
     const uint64_t start = global_ns();
     while (global_ns() - start < kDrainNs)
-        if (mbar_try_wait(bar, parity)) return;
+        if (mbar_try_wait<CG>(bar, parity)) return;
 }
 
 // ---------------------------------------------------------------- epilogue state
@@ -395,8 +408,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int rank = CG == 1 ? 0 : static_cast<int>(cluster_rank());
     const int unit = static_cast<int>(blockIdx.x) / CG;  // CTA or pair
     const int rt = unit / a.splits * CG + rank, split = unit % a.splits;
-    const int col_begin = static_cast<int>(lm_range(split, a.n_gran, a.splits, Sh::granule));
-    const int64_t col_end = lm_range(split + 1, a.n_gran, a.splits, Sh::granule);
+    const int col_begin = static_cast<int>(lm_range(split, a.n_gran, a.splits, a.granule));
+    const int64_t col_end = lm_range(split + 1, a.n_gran, a.splits, a.granule);
     const int n_tiles = static_cast<int>((col_end - col_begin + kTileN - 1) / kTileN);
     const int kblocks = a.d / kTileK;
     // With fewer rows than a tile the hidden copies are that high: filling most of
@@ -469,7 +482,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                                      static_cast<int64_t>(off) * kTileK * 2;
                 const int64_t next_blk = static_cast<int64_t>(kblocks) * kBBytes - static_cast<int64_t>(off) * kTileK * 2;
                 for (int kb = 0; kb < kblocks; kb += slices) {
-                    if (!wait_or_abort(&c.empty[s], ph ^ 1, c, a)) {
+                    if (!wait_or_abort<CG>(&c.empty[s], ph ^ 1, c, a)) {
                         ok = false;
                         break;
                     }
@@ -489,8 +502,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                                 blk += kBBytes;
                             } else if (n_cols == kTileN) {
                                 tma_load_2d(sb, &tm_w, (kb + j) * kTileK, col0, bar);
-                            } else {  // (tm_w_half: a granule per copy)
-                                for (int g = 0; g < n_cols; g += Sh::granule)
+                            } else {  // (tm_w_half: kCopyRows a copy)
+                                for (int g = 0; g < n_cols; g += kCopyRows)
                                     tma_load_2d(sb + g * (kTileK * 2), &tm_w_half, (kb + j) * kTileK, col0 + g, bar);
                             }
                             sa += a_bytes;
@@ -526,7 +539,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             // second CTA of a pair sees it by its stages being consumed.
             const uint32_t ring_len = n_stages;
             for (uint32_t j = it > ring_len ? it - ring_len : 0; j < it; ++j)
-                wait_drain(rank == 0 ? &c.full[j % ring_len] : &c.empty[j % ring_len], (j / ring_len) & 1);
+                wait_drain<CG>(rank == 0 ? &c.full[j % ring_len] : &c.empty[j % ring_len], (j / ring_len) & 1);
         }
     } else if (warp == 1) {
         if (lane == 0 && rank == 0) {  // --------------------------- MMA issuer
@@ -537,7 +550,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int t = 0; t < n_tiles && ok; ++t) {
                 const int buf = t & 1;
                 const uint32_t use = static_cast<uint32_t>(t >> 1);
-                if (!wait_or_abort(&c.acc_empty[buf], (use & 1) ^ 1, c, a)) break;
+                if (!wait_or_abort<CG>(&c.acc_empty[buf], (use & 1) ^ 1, c, a)) break;
                 tc_fence_after();
                 const uint32_t d_tmem = tmem + static_cast<uint32_t>(buf * kTileN);
                 const int n_cols = static_cast<int>(min(static_cast<int64_t>(kTileN), col_end - (col_begin + t * kTileN)));
@@ -545,7 +558,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const int slices = FLEX ? tile_slices(n_cols, a_bytes, stage_bytes) : Sh::slices;
                 const uint32_t a_step = a_bytes / 16, b_step = n_cols / CG * kTileK * 2 / 16, b_off = slices * a_step;
                 for (int kb = 0; kb < kblocks; kb += slices) {
-                    if (!wait_or_abort(&c.full[s], ph, c, a)) {
+                    if (!wait_or_abort<CG>(&c.full[s], ph, c, a)) {
                         ok = false;
                         break;
                     }
@@ -575,7 +588,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
             // every MMA issued has completed before TMEM is freed
             mma_commit<CG>(&c.mma_done);
-            wait_drain(&c.mma_done, 0);
+            wait_drain<CG>(&c.mma_done, 0);
         }
         __syncwarp();
     } else {  // ---------------------------------------------------- epilogue
@@ -599,7 +612,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int t = 0; t < n_tiles; ++t) {
             const int buf = t & 1;
             const uint32_t use = static_cast<uint32_t>(t >> 1);
-            if (!warp_wait_or_abort(&c.acc_full[buf], use & 1, c, a)) {
+            if (!warp_wait_or_abort<CG>(&c.acc_full[buf], use & 1, c, a)) {
                 ok = false;
                 break;
             }
@@ -737,7 +750,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     if constexpr (CG == 2) {
         // neither CTA leaves while the other's copies, MMAs or arrivals may reach
         // it: the last commit arrives in both
-        if (rank != 0 && threadIdx.x == 0 && !c.skip) wait_drain(&c.mma_done, 0);
+        if (rank != 0 && threadIdx.x == 0 && !c.skip) wait_drain<CG>(&c.mma_done, 0);
         __syncwarp();
         cluster_sync();
         __syncwarp();
@@ -1100,7 +1113,7 @@ struct LmLayout {
 // Splits the workspace is laid out for. One row tile takes every SM, also with
 // fewer vocabulary tiles than SMs.
 int64_t splits_cap(int32_t n_rows, int64_t vocab) {
-    const int tokens = n_rows <= kTileM ? Shape<1>::granule : kTileN;
+    const int tokens = n_rows <= kTileM ? kQuarter : kTileN;
     return std::min<int64_t>((vocab + tokens - 1) / tokens, kMaxSplits);
 }
 
@@ -1182,7 +1195,7 @@ rps_status rps_lmhead_row_stats(const rps_lmhead *lm, const rps_params *prm, con
     const int n_rt = (lm->n_rows + kTileM - 1) / kTileM;
     const int kblocks = lm->d / kTileK;
     const int64_t packed_blocks = static_cast<int64_t>(n_vt) * kblocks;
-    const LmSplit sp = lm_split(n_rt, lm->vocab, packed_blocks, cap, dev.sm_count, dev.pairs);
+    const LmSplit sp = lm_split(n_rt, lm->vocab, kblocks, cap, dev.sm_count, dev.pairs);
     const bool pair = sp.pair;
     const int units = sp.units, granule = sp.granule, n_gran = sp.n_gran, splits = sp.splits, longest = sp.longest;
     LmMaps maps;
@@ -1202,7 +1215,7 @@ rps_status rps_lmhead_row_stats(const rps_lmhead *lm, const rps_params *prm, con
         maps.w = maps.w_half = maps.h;  // (single CTAs read the packed unembedding without a tensor map)
         for (int part = 0; part < 2 && !lm->unembed_packed && st == RPS_OK; ++part)
             st = make_map(part ? &maps.w_half : &maps.w, lm->unembed, lm->vocab, lm->d, lm->unembed_stride,
-                          part ? Shape<1>::granule : kTileN);
+                          part ? kCopyRows : kTileN);
         if (st != RPS_OK) return st;
     }
 
@@ -1234,6 +1247,7 @@ rps_status rps_lmhead_row_stats(const rps_lmhead *lm, const rps_params *prm, con
     a.topk_logit = out->topk_logit;
 
     const cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+    a.granule = granule;
     a.n_gran = n_gran;
     // A single CTA's ring by its rows (FLEX), where that gives a fifth stage or
     // several slices in the last tile's stages; otherwise its code only costs (607

@@ -79,13 +79,16 @@ def check(h_bits, w_bits, k, rows=None):
 
 
 @pytest.mark.parametrize("n,d,V,k", [
-    (129, 64, 516, 10),      # a pair with one row in its second half, one K slice, a four-token granule
-    (256, 320, 40000, 10),   # whole row tiles; ranges that end in half a vocabulary tile
-    (260, 192, 40004, 32),   # an odd number of row tiles: the last pair's second half is empty
+    (129, 64, 516, 10),      # one K slice: too short for pairs
+    (129, 2112, 900, 10),    # a pair with one row in its second half, 33 K slices, a four-token granule
+    (256, 320, 40000, 10),   # five K slices: too short
+    (256, 1088, 40000, 10),  # whole row tiles; ranges that end in half a vocabulary tile
+    (260, 192, 40004, 32),   # three row tiles of single CTAs
+    (780, 1088, 9720, 20),   # an odd number of row tiles: the last pair's second half is empty
     (700, 128, 126464, 0),   # three pairs, several tiles each
 ])
 def test_lmhead_pairs(n, d, V, k):
-    """Two row tiles or more: a pair of CTAs per tile. Row-major and packed unembedding alike."""
+    """Two row tiles or more: a pair of CTAs per tile where that pays. Row-major and packed unembedding alike."""
     h, w = synth.lmhead_inputs(19, n, V, d)
     rows = np.unique(np.r_[0, 127, 128, n - 1, np.linspace(0, n - 1, 24).astype(int)])
     check(h, w, k, rows=rows)
@@ -122,7 +125,8 @@ def test_lmhead_merge_lists(n, V, k, zero):
     (33, 192, 40116, 0),     # ranges of five: a tile over two packed blocks, and one granule
     (128, 128, 60000, 10),   # ranges of seven: a tile and three granules
     (20, 2112, 9000, 10),    # ranges of one granule: four slices of d per stage, one left over
-    (300, 64, 20004, 10),    # three row tiles of single CTAs
+    (300, 64, 20004, 10),    # three row tiles of single CTAs, ranges of seven granules
+    (260, 64, 126300, 10),   # the same of whole tiles, the last one ragged
 ])
 def test_lmhead_ranges(n, d, V, k):
     """Vocabulary ranges of whole 64-token granules, row-major and packed alike; a workspace of
