@@ -62,11 +62,13 @@ inline LmSplit lm_cut(bool pair, int n_row_tiles, int granule, int64_t vocab, in
 // fit the ranges less well; an odd row tile makes a pair with an empty half; and a
 // launch of clusters takes longer (0.9 us in a graph, 4 us called directly). So pairs
 // take an even number of row tiles whose longest range is at most 1.2 times the
-// single CTAs', or an odd one from seven on (below 1.1), and longer than 32 slices.
+// single CTAs', or an odd one from seven on (1.12, 1.09 below 16 tiles), and longer
+// than 32 slices.
 // Best single against pairs, statistics only, us: d 4,096, 512 rows of V 126,464 341 /
 // 316, of V 8,000 31.8 / 31.1 (d 1,024: 17.4 / 21.0); 384 rows of V 126,464 297 / 332;
 // 1,152 rows of V 126,464 (1.06) 815 / 794, of V 20,000 (1.1) 4 % slower, of V 8,000 (1.25)
-// 54 / 65; 1,408 rows of V 126,464 (1.09), d 2,048 480 / 449.
+// 54 / 65; 1,408 rows of V 126,464 (1.09), d 2,048 480 / 449; 896 rows of V 90,000 to 134,348
+// (1.12) 3 % faster in pairs.
 // (The packed unembedding's blocks are tensor coordinates in a pair, 32 bits.)
 inline LmSplit lm_split(int n_row_tiles, int64_t vocab, int kblocks, int64_t cap, int sm_count, int pairs) {
     const LmSplit tiles = lm_cut(false, n_row_tiles, kTileN, vocab, cap, sm_count);
@@ -80,8 +82,8 @@ inline LmSplit lm_split(int n_row_tiles, int64_t vocab, int kblocks, int64_t cap
         const LmSplit p = lm_cut(true, n_row_tiles, kTileN / 2, vocab, cap, pairs);
         const int64_t pair_long = static_cast<int64_t>(p.longest) * p.granule;
         const int64_t single_long = cut ? quarters_long : tiles_long;
-        const bool fits = odd ? 10 * pair_long < 11 * single_long : 10 * pair_long <= 12 * single_long;
-        if (fits && pair_long * kblocks > 32 * kTileN) return p;
+        const int limit = !odd ? 120 : pair_long >= 16 * kTileN ? 112 : 109;
+        if (100 * pair_long <= limit * single_long && pair_long * kblocks > 32 * kTileN) return p;
     }
     return cut ? quarters : tiles;
 }

@@ -14,10 +14,10 @@ PROGRAM = r"""
 #include "lmhead_split.h"
 using namespace rps;
 int main() {
-    const int row_tiles[] = {1, 2, 2, 3, 3, 4, 5, 9, 9, 9, 11, 9, 2, 2, 7, 6, 3, 3};
-    const long long vs[] = {126464, 126464, 8000, 126464, 32000, 126464, 126464, 126464, 8000, 300, 126464, 20000, 900, 40000, 9720, 126464, 20004, 126300};
-    const int ds[] = {4096, 4096, 1024, 4096, 1024, 4096, 4096, 4096, 4096, 4096, 1024, 4096, 2112, 1088, 1088, 128, 64, 64};
-    for (int i = 0; i < 18; ++i) {
+    const int row_tiles[] = {1, 2, 2, 3, 3, 4, 5, 9, 9, 9, 11, 9, 2, 2, 7, 6, 3, 3, 7};
+    const long long vs[] = {126464, 126464, 8000, 126464, 32000, 126464, 126464, 126464, 8000, 300, 126464, 20000, 900, 40000, 9720, 126464, 20004, 126300, 90000};
+    const int ds[] = {4096, 4096, 1024, 4096, 1024, 4096, 4096, 4096, 4096, 4096, 1024, 4096, 2112, 1088, 1088, 128, 64, 64, 4096};
+    for (int i = 0; i < 19; ++i) {
         const LmSplit s = lm_split(row_tiles[i], vs[i], ds[i] / 64, row_tiles[i] == 1 ? 256 : std::min(256ll, (vs[i] + 255) / 256), 152, 76);
         std::printf("R %d %lld %d %d %d %d\n", row_tiles[i], vs[i], ds[i], s.pair, s.granule, s.splits);
     }
@@ -89,6 +89,7 @@ def test_forms(lines):
         (2, 900, 2112): (1, 128, 4),
         (2, 40000, 1088): (1, 128, 63),
         (7, 9720, 1088): (1, 128, 19),
+        (7, 90000, 4096): (1, 128, 19),    # 19 tiles against 17
         (6, 126464, 128): (1, 128, 25),
         (3, 20004, 64): (0, 64, 45),
         (3, 126300, 64): (0, 256, 50),
