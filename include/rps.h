@@ -304,9 +304,10 @@ rps_status rps_score_and_commit(const rps_logits *anchor_logits, int32_t anchor_
  * d_ws_branch, a different one), and rps_score_and_commit with branch 0 as the
  * anchor -- five launches with the results of the four calls. Every argument
  * is checked before anything is enqueued. Because the call knows which launch
- * writes what, the select launch stages the mask before waiting for the base
- * statistics, and the score launch computes everything that does not read the
- * lookahead statistics before waiting for them.
+ * writes what, the select launch stages the mask and takes the standard commit
+ * before waiting for the base rows' top-k search (unless the mask lies in an
+ * array of `piv` that it writes), and the score launch computes everything that
+ * does not read the lookahead statistics before waiting for them.
  */
 rps_status rps_run_step(const rps_logits *logits, int32_t n_req, int32_t L, const int32_t *d_mask_pos,
                         const int32_t *d_mask_cnt, const rps_params *prm, const rps_row_stats *base,

@@ -321,6 +321,21 @@ rps_status rps_select_pivots(const rps_row_stats *base, int32_t n_req, int32_t L
 namespace rps {
 namespace {
 
+// True when the mask lies in an array that select_request writes before its wait.
+bool mask_overlaps_select(const int32_t *mask_pos, const int32_t *mask_cnt, int32_t n_req, int32_t L,
+                          const rps_pivots &o) {
+    const size_t n = static_cast<size_t>(n_req), list = n * static_cast<size_t>(L);
+    const auto overlap = [](const int32_t *a, size_t na, const int32_t *b, size_t nb) {
+        const auto ua = reinterpret_cast<uintptr_t>(a), ub = reinterpret_cast<uintptr_t>(b);
+        return ua < ub + nb * sizeof(int32_t) && ub < ua + na * sizeof(int32_t);
+    };
+    for (const int32_t *w : {o.commit_pos, o.rem_k, o.rem_pos})
+        if (overlap(mask_pos, list, w, list) || overlap(mask_cnt, n, w, list)) return true;
+    for (const int32_t *w : {o.n_commit, o.rem_cnt, o.n_branch_rows})
+        if (overlap(mask_pos, list, w, n) || overlap(mask_cnt, n, w, n)) return true;
+    return false;
+}
+
 rps_status make_score_args(const rps_logits *anchor_logits, int32_t anchor_branch, const rps_row_stats *anchor,
                            const rps_row_stats *branch, int32_t n_req, int32_t L, const rps_pivots *piv,
                            const rps_params *prm, const rps_branch_scores *out, ScoreArgs *a) {
@@ -471,8 +486,9 @@ rps_status rps_run_step(const rps_logits *logits, int32_t n_req, int32_t L, cons
     if (d_ws_base == d_ws_branch) return RPS_ERR_INVALID_ARG;
     sc.err = a_la.err;
     // inside one step the select launch follows the base statistics only, and
-    // score and commit follow the lookahead statistics only
-    sel.early = 1;
+    // score and commit follow the lookahead statistics only. (Select writes M' and
+    // the commit set's positions while the top-k search may still read the mask.)
+    sel.early = !mask_overlaps_select(d_mask_pos, d_mask_cnt, n_req, L, *piv);
     sc.early = 1;
     const cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     cudaError_t e = launch_row_stats(a_base, logits->dtype, grid_base, topk_grid_base, s);

@@ -85,3 +85,30 @@ def test_tiny_vocabularies(V, bf16):
     if V == 1:
         assert np.allclose(out["base"].H[[0, 1, 2]], 0.0, atol=1e-6) and np.allclose(out["base"].pmax[[0, 1, 2]], 1.0)
         assert (out["piv"]["state"] == 1).all(), "a single-token vocabulary commits everything"
+
+
+@pytest.mark.parametrize("pos_in,cnt_in", [("rem_pos", "rem_cnt"), ("commit_pos", "n_commit"), ("rem_pos", None),
+                                           (None, "rem_cnt")])
+def test_mask_in_an_array_that_select_writes(pos_in, cnt_in):
+    """A step whose mask lies in one of its outputs: select may not write there while the
+    top-k search still reads the mask (more slots than the search takes in one round)."""
+    n, L, V = 64, 512, 64
+    prm = Params(8, 0.1, 0.05, 0.6, 1.0, 1, 2)
+    g = torch.Generator(device="cuda").manual_seed(3)
+    z = 3.0 * torch.randn((n, 3, L, V), generator=g, device="cuda")
+    pos = torch.stack([torch.randperm(L, generator=g, device="cuda") for _ in range(n)]).int().sort(1).values.contiguous()
+    cnt = torch.full((n,), L, dtype=torch.int32, device="cuda")
+    want = rps.Step(n, L, V, prm, "cuda", z.dtype)
+    want.run(z, pos, cnt)
+    got = rps.Step(n, L, V, prm, "cuda", z.dtype)
+    p = pos if pos_in is None else getattr(got.piv, pos_in).copy_(pos.view_as(getattr(got.piv, pos_in)))
+    c = cnt if cnt_in is None else getattr(got.piv, cnt_in).copy_(cnt)
+    got.run(z, p, c)
+    assert rps.rps_poll_device_status() == (rps.RPS_OK, 0)
+    assert int(want.piv.rem_cnt.sum()) > 0 and int(want.piv.n_commit.sum()) > 0
+    for f in ("argmax", "mu", "topk_idx", "H"):
+        assert torch.equal(getattr(got.base, f), getattr(want.base, f)), f
+    for f in ("n_commit", "rem_cnt", "state", "pivot_pos", "n_branch_rows"):
+        assert torch.equal(getattr(got.piv, f), getattr(want.piv, f)), f
+    for f in ("winner", "commit_pos", "mask_cnt"):
+        assert torch.equal(getattr(got.commit, f), getattr(want.commit, f)), f
