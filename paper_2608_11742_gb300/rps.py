@@ -239,7 +239,6 @@ class RowStatsBuf(_CStruct):
         return RowStatsBuf(f(n), f(n), f(n), f(n), i(n))
 
 
-
 @dataclass
 class PivotsBuf(_CStruct):
     n_commit: torch.Tensor
@@ -269,7 +268,6 @@ class PivotsBuf(_CStruct):
                          i(n_req), i(n_req, NB * L, 3))
 
 
-
 @dataclass
 class ScoresBuf(_CStruct):
     mean_H: torch.Tensor
@@ -281,7 +279,6 @@ class ScoresBuf(_CStruct):
     def alloc(n_req: int, P: int, K: int, device) -> "ScoresBuf":
         f = lambda: torch.full((n_req, P, K + 1), float("nan"), dtype=torch.float32, device=device)
         return ScoresBuf(f(), torch.full((n_req, P, K + 1), -1, dtype=torch.int32, device=device), f(), f())
-
 
 
 @dataclass
@@ -302,7 +299,6 @@ class CommitBuf(_CStruct):
         return CommitBuf(i(n_req, P), f(n_req, P), i(n_req), i(n_req), i(n_req), f(n_req), i(n_req, L), i(n_req))
 
 
-
 for _cls, _st in ((RowStatsBuf, RpsRowStats), (PivotsBuf, RpsPivots), (ScoresBuf, RpsBranchScores),
                   (CommitBuf, RpsCommitOut)):
     _cls._struct = _st
@@ -310,8 +306,8 @@ for _cls, _st in ((RowStatsBuf, RpsRowStats), (PivotsBuf, RpsPivots), (ScoresBuf
 
 
 def _cs(buf):
-    """The C struct of a buffer set (any object with ``c()`` will do)."""
-    return buf._c() if isinstance(buf, _CStruct) else buf.c()
+    """The C struct of a buffer set (any object with ``c()`` will do; a subclass's own is called)."""
+    return buf._c() if type(buf).c is _CStruct.c else buf.c()
 
 
 # --------------------------------------------------------------------------- ABI calls

@@ -39,3 +39,21 @@ def test_kept_struct_follows_the_tensors(make):
     assert addresses(buf) == expected(buf, names)
     for other in (copy.copy(buf), copy.deepcopy(buf), pickle.loads(pickle.dumps(buf))):
         assert addresses(other) == expected(other, names)
+
+
+def test_a_subclass_may_form_its_own_struct():
+    """``c()`` of a subclass is what the calls pass on."""
+    class Own(rps.ScoresBuf):
+        def c(self):
+            return rps.RpsBranchScores(64, 2, 3, 4)
+
+    class Other:
+        def c(self):
+            return rps.RpsBranchScores(1, 2, 3, 4)
+
+    name = rps.RpsBranchScores._fields_[0][0]
+    plain = rps.ScoresBuf.alloc(2, 3, 2, "cpu")
+    own = Own(*(getattr(plain, n) for n, _ in rps.RpsBranchScores._fields_))
+    assert getattr(rps._cs(own), name) == 64
+    assert getattr(rps._cs(Other()), name) == 1
+    assert getattr(rps._cs(plain), name) == getattr(plain, name).data_ptr()
