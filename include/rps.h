@@ -461,7 +461,10 @@ rps_status rps_lmhead_row_stats(const rps_lmhead *lm, const rps_params *prm, con
  * normal sequence). For every (batch, head):
  *   out_i = sum_{k visible from i} softmax_k(scale * q_i . k_k) v_k
  * bf16 inputs and output, fp32 scores and accumulation, probabilities rounded
- * to bf16 before they weight the values. No dense mask is formed.
+ * to bf16 before they weight the values. No dense mask is formed. Scores of
+ * -inf take no weight. The values must be finite: keys that a query does not
+ * see weigh nothing, but they may share a tile with keys that it sees, where a
+ * value of inf or NaN makes the output NaN.
  * Layout (bf16, contiguous): q, k, out [n_batch][n_heads][n_tokens][head_dim];
  * vt [n_batch][n_heads][head_dim][n_tokens] (the values transposed, tokens
  * contiguous). head_dim must be 128; n_context (>= 0) and branch_len (>= 1)

@@ -776,8 +776,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
                 l *= f;
                 // P = 2^(s c - m) (a masked key gives 2^-inf = 0), bf16 pairs, over
-                // the first 64 columns of S (already in registers)
-                const f2 cc = pack2(a.c, a.c), mm = pack2(-m, -m);
+                // the first 64 columns of S (already in registers). Scores of -inf in
+                // all of the half's tiles so far leave m there: P = 0, and the sum 0.
+                const float mr = m == -INFINITY ? 0.f : -m;
+                const f2 cc = pack2(a.c, a.c), mm = pack2(mr, mr);
                 f2 lsum[4] = {pack2(0.f, 0.f), pack2(0.f, 0.f), pack2(0.f, 0.f), pack2(0.f, 0.f)};
                 uint32_t pk[32];
                 exp_scores(s0, cc, mm, lsum, pk, 0);
