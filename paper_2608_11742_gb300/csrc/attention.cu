@@ -38,15 +38,16 @@
 //   warps 12-15 read-out: at the end of an item the halves' accumulators are
 //               weighted by 2^(m_half - m) / l, added and written as bf16, while the
 //               softmax goes on with the next item.
-// Bound by the MMA issue: the 16 instructions of a key tile take 1,024 cycles of
-// work, and each commit costs their thread about 200 that instructions of N 128
-// do not hide: about 1,490 of the 2,050 cycles of a tile; the rest are its waits
-// (K, V, P, and the read-out at the items' ends). A half waits for S most of the
-// time: its softmax takes 1,330 to 1,540 cycles, and two run at once. Shared-memory
-// traffic is not the limit: pairs of CTAs that share K and V (160 -> 96 KB per tile)
-// took the same time. 8 x 32 heads, context 512, 9 branches of 256: 266 -> 254 us; 32
-// heads, context 328, 9 branches of 32: 20.4 -> 13.9 us (against two halves of each
-// row in turn with separate S and P V issuers, and a tile per branch).
+// What bounds it: the MMA issue and the issuer's waits, in turn. Of about 2,090 cycles
+// of a key tile the issuer spends 1,490 on its 16 instructions of N 128 (1,024 cycles of
+// work; back to back, batches of 16 with one commit take 1,230, each further commit
+// about 50) and 600 waiting: for the read-out at the items' ends 213, P 136, K 107, V 103,
+// Q 41. A half of the softmax waits for S most of the time: it takes 1,330 to 1,540
+// cycles, and two run at once. Shared-memory traffic is not the limit: pairs of CTAs
+// that share K and V (160 -> 96 KB per tile) took the same time. 8 x 32 heads, context
+// 512, 9 branches of 256: 262 -> 248 us; 32 heads, context 328, 9 branches of 32: 20.3 ->
+// 13.9 us (against two halves of each row in turn with separate S and P V issuers, and
+// a tile per branch).
 // Every wait is bounded; a role whose wait runs out flags RPS_DEVERR_TIMEOUT
 // and raises the CTA's abort flag, copies and MMAs in flight are drained and
 // TMEM is freed before the CTA exits.
@@ -387,8 +388,8 @@ struct Ctl {
     // tile t - 2 is done, so K stage t % 2 and Q of the items before t's are free.
     // V stage t % 2 has a commit of its own right after the product (v_empty):
     // its next tile is then on its way while S of tile t + 2 is computed, which
-    // is worth more than the commit's 50 cycles (8 x 32 heads, context 512, 9
-    // branches of 256: 258 -> 254 us). No wait sees a barrier two phases on: each
+    // is worth more than the 50 cycles of a second commit per tile (the first
+    // takes about 200; 8 x 32 heads, context 512, 9 branches of 256: 258 -> 254 us). No wait sees a barrier two phases on: each
     // waits for every phase in turn. (The read-out waits once an item, on a
     // barrier of its own: o_ready.)
     uint64_t q_full[kQBufs], k_full[kKvStages], v_full[kKvStages], v_empty[kKvStages];

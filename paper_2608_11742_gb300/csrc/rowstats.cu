@@ -1188,9 +1188,11 @@ __device__ __forceinline__ uint32_t cell_hits(const uint4 *sk, int v, float thet
 // FEW: rows of at most kFewChunks ring chunks. One sketch entry per lane and chunk fits
 // the registers, so the bound is taken over cells (each lane's largest two)
 // instead of vectors of them, and the hits need no second look. A short row has
-// too few vectors: V 3,447 has 16, so that at k = 32 every cell was reloaded (64
-// rows: 434 us, here 13; k = 16 at V 2,100 26.6 -> 10.8, k = 10 the same).
+// too few vectors that hold any (its pieces fill a chunk's first lanes only), so that
+// for long lists every cell was reloaded. 64 bf16 rows, k = 32, both launches: V 3,447
+// 516 -> 17 us, V 16,000 32.5 -> 16.3; k = 16, V 2,100 34 -> 14.
 static_assert(kFewChunks <= 32, "one hit bit per chunk");
+static_assert(sketch_entries(1) >= 32 * kFewChunks, "every slot holds that many chunks (-inf past the row's)");
 
 template <int DT, bool FEW>
 __global__ void __launch_bounds__(kTopkWarps * 32, kTopkMinBlocks) topk_rows_kernel(const RowStatsArgs a) {
@@ -1215,6 +1217,11 @@ __global__ void __launch_bounds__(kTopkWarps * 32, kTopkMinBlocks) topk_rows_ker
     const int n_vec = static_cast<int>(a.sketch_stride / kPerVec);  // the whole slot (-inf past the row's chunks)
     const bool one_batch = n_vec <= 32 * kSketchVecs;
     bool waited = false;
+    // FEW: this lane's cell of chunk c. A piece shorter than a chunk's 32 lanes fills
+    // the first ones only, so each chunk starts where the one before it ended:
+    // the row's cells go round all lanes.
+    const int turn = static_cast<int>(min(a.min_piece, static_cast<int64_t>(32)));
+    const auto few_cell = [&](int c) { return c * 32 + ((lane - c * turn) & 31); };
 
     // One warp per list slot (entry), in slot order: no scan of the list.
     for (int64_t slot = static_cast<int64_t>(blockIdx.x) * kTopkWarps + wib;;
@@ -1250,8 +1257,7 @@ __global__ void __launch_bounds__(kTopkWarps * 32, kTopkMinBlocks) topk_rows_ker
         if constexpr (FEW) {
             const typename E::Sketch *entries = reinterpret_cast<const typename E::Sketch *>(sk);
 #pragma unroll
-            for (int c = 0; c < kFewChunks; ++c)
-                em[c] = c * 32 < a.sketch_stride ? E::from_sketch(__ldg(entries + c * 32 + lane)) : -INFINITY;
+            for (int c = 0; c < kFewChunks; ++c) em[c] = E::from_sketch(__ldg(entries + few_cell(c)));
         } else {
             vector_maxima<DT>(vm, sk, 0, n_vec, lane);
         }
@@ -1314,14 +1320,14 @@ __global__ void __launch_bounds__(kTopkWarps * 32, kTopkMinBlocks) topk_rows_ker
             if (theta == -INFINITY) {  // (not the entries past the row's chunks)
                 for (uint32_t b = he; b; b &= b - 1) {
                     int first, count;
-                    sketch_cell(cut, full_units, (__ffs(b) - 1) * 32 + lane, first, count);
+                    sketch_cell(cut, full_units, few_cell(__ffs(b) - 1), first, count);
                     if (count == 0) he &= ~(b & (0u - b));
                 }
             }
             if (lane == 0) *n_cells = 0;
             __syncwarp();
             int at = he ? atomicAdd(n_cells, __popc(he)) : 0;
-            for (; he && at < kCellCap; he &= he - 1) cells[at++] = (__ffs(he) - 1) * 32 + lane;
+            for (; he && at < kCellCap; he &= he - 1) cells[at++] = few_cell(__ffs(he) - 1);
             __syncwarp();
             listed = *n_cells <= kCellCap;
             if (listed) pending = *n_cells;  // else in rounds, as vectors
