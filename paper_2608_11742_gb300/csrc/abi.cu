@@ -225,6 +225,14 @@ rps_status prepare_row_stats(const rps_logits *logits, const rps_row_list *rows,
                                                          static_cast<int64_t>(dev.sm_count) * 16));
     a.min_piece = (a.units_per_row + (kMaxPartials - 2) - 1) / (kMaxPartials - 2);
     a.max_ppr = static_cast<int32_t>((a.units_per_row + a.min_piece - 1) / a.min_piece);
+    // Few rows: a warp for each part of a row (max_ppr + 1 at most), while the aligned
+    // cut would idle more than an eighth of the warps. The pieces are then the
+    // shortest, whatever the row count. (32-bit arithmetic over all units.)
+    const int64_t longest = (a.units_per_row + a.max_ppr - 1) / a.max_ppr;  // of the aligned cut's pieces
+    const int64_t aligned = (a.units_per_row + longest - 1) / longest;      // and their number
+    a.few_rows = static_cast<int32_t>(std::min({static_cast<int64_t>(a.warps) / (a.max_ppr + 1),
+                                                (7 * static_cast<int64_t>(a.warps) - 1) / (8 * aligned),
+                                                ((int64_t{1} << 30) - 1) / a.units_per_row}));
     // The ring chunks of a row under any cut, whose n parts are at most one more
     // than the pieces of its length: one each while a piece fits a chunk, else at
     // most the row's whole chunks and n.

@@ -640,10 +640,11 @@ __device__ __forceinline__ void locate(const RowStatsArgs &a, const int32_t *seg
     describe<DT>(a, seg, s);
 }
 
-// a / b for 0 < b and a below 2^22, exact: the approximate quotient is off by at
-// most one, and the remainder says which way. A fifth of the instructions of an
-// integer division; the 32 warps of a block all compute the cut, in the same
-// issue slots, before the first copy can start.
+// a / b for 0 < b, exact for a below 2^22, or a + b below 2^31 and a quotient below
+// 2^20: the approximate quotient is off by at most one, and the remainder says
+// which way. A fifth of the instructions of an integer division; the 32 warps of a
+// block all compute the cut, in the same issue slots, before the first copy can
+// start, and after a forward pass its code comes from memory line by line.
 __device__ __forceinline__ int div_small(int a, int b) {
     int q = __float2int_rz(__fdividef(static_cast<float>(a), static_cast<float>(b)));
     const int r = a - q * b;
@@ -652,21 +653,24 @@ __device__ __forceinline__ int div_small(int a, int b) {
     return q;
 }
 
-// The cut of the rows' units into pieces. Aligned: each row is cut into `cpr`
-// equal pieces (at most a.max_ppr), so that no piece crosses a row boundary,
-// where a warp's stream stops for the row's record; taken when it leaves at most
-// an eighth of the warps idle. Otherwise all units are cut evenly, in pieces of at
-// least min_piece units, and cpr is 0. few: the pieces are that short and warps
-// are left over, enough for one per part of a row.
+// The cut of the rows' units into pieces. few (at most a.few_rows): pieces of
+// min_piece units, the shortest, laid end to end over the rows, and a warp for
+// each part of a row. Else aligned: each row is cut into `cpr` equal pieces (at
+// most a.max_ppr), so that no piece crosses a row boundary, where a warp's stream
+// stops for the row's record; taken when it leaves at most an eighth of the warps
+// idle. Otherwise all units are cut evenly, in pieces of at least min_piece units,
+// and cpr is 0.
 // The parts decide how a row's sums round, and scores that are equal in exact
 // arithmetic (a token and [MASK] over rows that are the same in their branches)
 // are told apart by that rounding. So this rule is part of the results: with
-// pieces of a ring chunk at least, or with the aligned cut also for rows of short
-// pieces (1,000 bf16 rows of V 9,807 16.1 -> 13.1 us), other slots win.
+// pieces of a ring chunk at least, or with the aligned cut also for few rows and
+// for rows of short pieces (1,000 bf16 rows of V 9,807 16.1 -> 13.1 us), other slots
+// win.
 __device__ __forceinline__ int64_t piece_units(const RowStatsArgs &a, int64_t total_rows, int64_t nv, int &cpr,
                                                bool &few) {
     cpr = 0;
-    few = false;
+    few = total_rows <= a.few_rows;
+    if (few) return a.min_piece;
     if (total_rows <= a.warps) {  // (rows, warps and units of a row fit 32 bits)
         const int rows = static_cast<int>(total_rows), n = static_cast<int>(nv);
         int piece, c;
@@ -683,8 +687,6 @@ __device__ __forceinline__ int64_t piece_units(const RowStatsArgs &a, int64_t to
             cpr = c;
             return piece;
         }
-        few = total_rows * nv <= (a.min_piece - 1) * a.warps && rows * (a.max_ppr + 1) <= a.warps;
-        if (few) return a.min_piece;
     }
     return max((total_rows * nv + a.warps - 1) / a.warps, a.min_piece);
 }
@@ -853,18 +855,16 @@ __global__ void __launch_bounds__(kStatThreads, kStatBlocksPerSm) row_stats_kern
         // crosses a row boundary goes to two warps, one for each row's part:
         // max_ppr + 1 places to a row. (With nearly all warps in use neighbouring
         // pieces stay in one block: spread, the 256-position step was 1.2 % slower.)
+        // Few instructions before the first copy, the parts' count after it: with
+        // code and data from memory the step 57.3 -> 53.3 us, of V 4,096 44.9 -> 40.3.
         const int w = wib * static_cast<int>(gridDim.x) + static_cast<int>(blockIdx.x);
         const int places = a.max_ppr + 1, row0 = div_small(w, places), part = w - row0 * places;
         if (row0 >= total_rows) return;
-        const int64_t begin = row0 * nv;
         const int len = static_cast<int>(piece), n = static_cast<int>(nv);
-        one.before = begin < (1 << 22)
-                         ? static_cast<int>(begin) - div_small(static_cast<int>(begin), len) * len
-                         : static_cast<int>(begin % len);
+        one.before = row0 * n - div_small(row0 * n, len) * len;
         const int from = max(part * len - one.before, 0), to = min((part + 1) * len - one.before, n);
         if (from >= to) return;
         one.mine = part;
-        one.parts = 1 + (n < (1 << 21) ? div_small(one.before + n - 1, len) : (one.before + n - 1) / len);
         w0.r = row0;
         w0.u = from;
         w0.left = to - from;
@@ -897,6 +897,9 @@ __global__ void __launch_bounds__(kStatThreads, kStatBlocksPerSm) row_stats_kern
         }
     }
     issued = __shfl_sync(kFull, issued, 0);
+    if (few && lane == 0)
+        one_row[wib].parts = 1 + div_small(one_row[wib].before + static_cast<int>(nv) - 1, static_cast<int>(piece));
+    __syncwarp();
     int acquired = 0, released = 0;
 
     // Waits for the next ring chunk; false when it does not land within the

@@ -86,6 +86,7 @@ struct RowStatsArgs {
     int64_t min_piece;    // at least ceil(units_per_row / (kMaxPartials - 1))
     int32_t few_chunks;   // no cut leaves a row more than kFewChunks ring chunks (top-k mode)
     int32_t max_ppr;      // ceil(units_per_row / min_piece): pieces a row is cut into at most
+    int32_t few_rows;     // up to this many rows a warp takes one part of one row
     uint32_t *err;
 };
 
